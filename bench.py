@@ -233,11 +233,15 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
          {"fp64": "fp64", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "tf32"}[prec]),
         ("interp_" + suffix, float(n) * df_interp_inst(K) if prec == "df64" else fl_in,
          {"fp64": "fp64", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "fp32"}[prec]),
+        # FP64 and DF64 plans: 27 digit products per 8 orders, m16n8k16, 8 samples a group
+        ("interp_fx", float(n) * 27 * 2 * 16 * 16 * ((K + 7) // 8), "fp16"),
     ]
     peaks = {"fp64": (PEAK_FP64_TFLOPS, "TFLOP/s", "alu", "derived: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz"),
              "fp32": (PEAK_FP32_TFLOPS, "TFLOP/s", "alu", "derived: 152 SMs x 128 FFMA/clk x 2 flops x 2.07 GHz"),
              "fp32inst": (PEAK_FP32_TINST, "Tinst/s", "alu",
                           "derived: 152 SMs x 128 FP32 instructions/clk x 2.07 GHz (double-float arithmetic)"),
+             "fp16": (float(measured_peaks().get("bf16_tflops", 1900.0)), "TFLOP/s", "tensor",
+                      "measured bf16 burst (MEASURED_PEAKS.json); digit products of full groups"),
              "tf32": (PEAK_TF32_TFLOPS, "TFLOP/s", "tensor",
                       "measured bf16 burst (MEASURED_PEAKS.json) x nominal TF32/BF16 ratio 1.1/2.25 (of measured)")}
     roofs = {}
@@ -265,6 +269,7 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
     cube_bytes = float(R) * nphi * (K + 1) * elem
     alg_bytes = {lc_name: float(ncomp) * plan.nalm * 16 * 2 + (K + 1) * R * (2 * L + 1) * elem,
                  "interp_" + suffix: n * (8.0 + 8.0 + (24.0 if elem == 16 else 16.0) + 4.0) + cube_bytes}
+    alg_bytes["interp_fx"] = alg_bytes["interp_" + suffix]
     for name, r in roofs.items():
         if name in alg_bytes:
             sec = r["avg_ms"] / 1e3

@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "interp_f64.cuh"
 #include "mbar.cuh"
 #include "sl_internal.cuh"
 
@@ -29,7 +30,8 @@ namespace sl {
 constexpr int kChunkA = kWorkChunk;
 
 // ------------------------------------------------------------------ forward FP64
-// One thread per sample: combined weights w_a w_b per node, read through L1.
+// One thread per sample: for a sort by tile (interp_tod_noalloc), where the samples of a
+// cell are not adjacent, and where interp_uses_fx finds the cell products no faster.
 template <int P>
 __global__ void __launch_bounds__(256) k_interp_f64(const InterpGeom g, const double2 *__restrict__ maps,
                                                     const StencilRec64 *__restrict__ rec,
@@ -37,60 +39,7 @@ __global__ void __launch_bounds__(256) k_interp_f64(const InterpGeom g, const do
                                                     int64_t n, double *__restrict__ tod) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const unsigned s = perm[t];
-        const StencilRec64 r = rec[s];
-        const int i = (int)(r.cell >> 16) - 1, j = (int)(r.cell & 0xffffu);
-        double wt[P], wp[P];
-        weights64<P>(g, i, r.dth, r.fph, wt, wp);
-        int roff[P], coff[P], coffg[P];
-        const unsigned ghost = stencil_offsets<P>(g, i, j, roff, coff, coffg);
-        // node offsets and combined weights (ghost rows read the ring at phi + pi)
-        int off[P * P];
-        double w[P * P];
-#pragma unroll
-        for (int a = 0; a < P; ++a)
-#pragma unroll
-            for (int b = 0; b < P; ++b) {
-                off[a * P + b] = roff[a] + (((ghost >> a) & 1u) ? coffg[b] : coff[b]);
-                w[a * P + b] = wt[a] * wp[b];
-                if (!SL_GUARD(off[a * P + b] >= 0 &&
-                                  (int64_t)off[a * P + b] + g.K < (int64_t)g.R * g.nphi * (g.K + 1),
-                              0x201u))
-                    off[a * P + b] = 0;
-            }
-        double sp, cp;
-        sincos(psi[s], &sp, &cp);
-        // k = 0: only Re S_0 enters the TOD
-        double acc = 0.0;
-#pragma unroll
-        for (int q = 0; q < P * P; ++q) acc = fma(w[q], __ldg(maps + off[q]).x, acc);
-        // C_k = 2 cos(k psi), S_k = 2 sin(k psi) by the Chebyshev three-term
-        // recurrence X_{k+1} = (2 cos psi) X_k - X_{k-1}
-        const double c1 = 2.0 * cp;
-        double Ck = c1, Sk = 2.0 * sp, Ckm = 2.0, Skm = 0.0;
-        for (int k = 1; k <= g.K; ++k) {
-            if (ghost) {   // (-1)^k on ghost rows: flip their weights between k-1 and k
-#pragma unroll
-                for (int a = 0; a < P; ++a)
-                    if (ghost & (1u << a))
-#pragma unroll
-                        for (int b = 0; b < P; ++b) w[a * P + b] = -w[a * P + b];
-            }
-            double sr = 0.0, si = 0.0;
-#pragma unroll
-            for (int q = 0; q < P * P; ++q) {
-                const double2 v = __ldg(maps + off[q] + k);
-                sr = fma(w[q], v.x, sr);
-                si = fma(w[q], v.y, si);
-            }
-            acc = fma(Ck, sr, acc);
-            acc = fma(-Sk, si, acc);
-            const double cn = fma(c1, Ck, -Ckm), sn = fma(c1, Sk, -Skm);
-            Ckm = Ck;
-            Skm = Sk;
-            Ck = cn;
-            Sk = sn;
-        }
-        tod[s] = acc;
+        tod[s] = interp_one_f64<P>(g, maps, rec[s], psi[s]);
     }
 }
 
@@ -899,22 +848,33 @@ sl_status launch_interp_f32_cells(cudaStream_t stream, int device, const TiledAr
     return cuda_check(cudaGetLastError(), "k_interp_f32_cells launch");
 }
 
+static sl_status launch_interp_f64(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n,
+                                   double *tod) {
+    void (*kern)(const InterpGeom, const double2 *, const StencilRec64 *, const double *, const unsigned *, int64_t,
+                 double *);
+    switch (p->p) {
+        case 2: kern = k_interp_f64<2>; break;
+        case 4: kern = k_interp_f64<4>; break;
+        case 6: kern = k_interp_f64<6>; break;
+        default: return set_error(SL_ERR_UNSUPPORTED, "interp_order %d", p->p);
+    }
+    const int slot = timing_begin(p, "interp_f64");
+    kern<<<grid_for(n, 256), 256, 0, p->stream>>>(p->geom, (const double2 *)maps, (const StencilRec64 *)b.rec, psi,
+                                                  b.perm, n, tod);
+    timing_end(p, slot);
+    return cuda_check(cudaGetLastError(), "k_interp_f64 launch");
+}
+
+int interp_needs_chunks(const sl_plan *p, int64_t n_total) {
+    return plan_fp32(p->precision) || (p->precision == SL_DF64 && !interp_uses_fx(p, n_total));
+}
+
 sl_status launch_interp(sl_plan *p, const SortBufs &b, int fine, const void *maps, const double *psi, int64_t n,
-                        double *tod) {
-    int slot;
+                        int64_t n_total, double *tod) {
+    if (fine && interp_uses_fx(p, n_total)) return launch_interp_fx(p, b, maps, psi, n, tod);
     if (p->precision == SL_DF64) return launch_interp_df(p, b, fine, maps, psi, n, tod);
     if (p->precision == SL_FP64) {
-        void (*kern)(const InterpGeom, const double2 *, const StencilRec64 *, const double *, const unsigned *,
-                     int64_t, double *);
-        switch (p->p) {
-            case 2: kern = k_interp_f64<2>; break;
-            case 4: kern = k_interp_f64<4>; break;
-            case 6: kern = k_interp_f64<6>; break;
-            default: return set_error(SL_ERR_UNSUPPORTED, "interp_order %d", p->p);
-        }
-        slot = timing_begin(p, "interp_f64");
-        kern<<<grid_for(n, 256), 256, 0, p->stream>>>(p->geom, (const double2 *)maps, (const StencilRec64 *)b.rec,
-                                                       psi, b.perm, n, tod);
+        return launch_interp_f64(p, b, maps, psi, n, tod);
     } else {
         if (!b.chunk_off) return set_error(SL_ERR_ARG, "FP32 interpolation needs the per-tile work list");
         TiledArgs a;
@@ -929,7 +889,7 @@ sl_status launch_interp(sl_plan *p, const SortBufs &b, int fine, const void *map
         a.tod = tod;
         if (fine) {   // cell-sorted samples: S samples of a cell per thread
             if (!p->d_err) return set_error(SL_ERR_ARG, "FP32 interpolation needs the plan's error flag");
-            slot = timing_begin(p, "interp_f32");
+            const int slot = timing_begin(p, "interp_f32");
             sl_status st = launch_interp_f32_cells(p->stream, p->device, &a, 1, p->geom.tile_cols, p->p, p->K,
                                                    reinterpret_cast<unsigned *>(p->d_err + 1), p->d_err);
             timing_end(p, slot);
@@ -951,10 +911,10 @@ sl_status launch_interp(sl_plan *p, const SortBufs &b, int fine, const void *map
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, sm);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
         if (per_sm < 1) per_sm = 1;
-        slot = timing_begin(p, "interp_f32");
+        const int slot = timing_begin(p, "interp_f32");
         kern<<<(unsigned)(nsm * per_sm), 256, sm, p->stream>>>(a);
+        timing_end(p, slot);
     }
-    timing_end(p, slot);
     return cuda_check(cudaGetLastError(), "k_interp launch");
 }
 

@@ -143,15 +143,18 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned &e
     return tot;
 }
 
-// Per CTA: exclusive scan of data[b*4096 .. +4096) in place, block total to bsum[b].
+// Per CTA: exclusive scan of data[b*4096 .. +4096) in place, block total to bsum[b], the
+// number of nonzero entries to nz[b].
 __global__ void __launch_bounds__(1024) k_scan_local(int64_t n, unsigned *__restrict__ data,
-                                                      unsigned *__restrict__ bsum) {
+                                                      unsigned *__restrict__ bsum, unsigned *__restrict__ nz) {
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + 4 * threadIdx.x;
     unsigned v[4], t = 0;
+    int nonzero = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         v[q] = (base + q < n) ? data[base + q] : 0u;
         t += v[q];
+        nonzero += __syncthreads_count(v[q] != 0u);
     }
     unsigned ex;
     const unsigned tot = block_exclusive_scan(t, ex);
@@ -160,12 +163,17 @@ __global__ void __launch_bounds__(1024) k_scan_local(int64_t n, unsigned *__rest
         if (base + q < n) data[base + q] = ex;
         ex += v[q];
     }
-    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
+    if (threadIdx.x == 0) {
+        bsum[blockIdx.x] = tot;
+        nz[blockIdx.x] = (unsigned)nonzero;
+    }
 }
 
-// Single CTA: exclusive scan of data[0..n) in place; data[n] = total.
-__global__ void __launch_bounds__(1024) k_scan1(int n, unsigned *__restrict__ data) {
-    unsigned carry = 0;
+// Single CTA: exclusive scan of data[0..n) in place; data[n] = total.  With occ, also
+// *occ = the sum of nz[0..n).
+__global__ void __launch_bounds__(1024) k_scan1(int n, unsigned *__restrict__ data, const unsigned *__restrict__ nz,
+                                                unsigned *__restrict__ occ) {
+    unsigned carry = 0, occupied = 0;
     for (int base = 0; base < n; base += 1024) {
         const int t = base + threadIdx.x;
         const unsigned v = (t < n) ? data[t] : 0u;
@@ -173,8 +181,12 @@ __global__ void __launch_bounds__(1024) k_scan1(int n, unsigned *__restrict__ da
         const unsigned tot = block_exclusive_scan(v, ex);
         if (t < n) data[t] = carry + ex;
         carry += tot;
+        if (occ) occupied += block_exclusive_scan((t < n) ? nz[t] : 0u, ex);
     }
-    if (threadIdx.x == 0) data[n] = carry;
+    if (threadIdx.x == 0) {
+        data[n] = carry;
+        if (occ) *occ = occupied;
+    }
 }
 
 __global__ void k_scan_add(int64_t n, unsigned *__restrict__ data, const unsigned *__restrict__ bsum,
@@ -299,8 +311,8 @@ sl_status launch_sort_into(sl_plan *p, const SortBufs &b, const double *theta, c
     timing_end(p, slot);
     if ((st = cuda_check(cudaGetLastError(), "k_bin launch")) != SL_OK) return st;
     slot = timing_begin(p, "scan");
-    k_scan_local<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum);
-    k_scan1<<<1, 1024, 0, p->stream>>>((int)nb, b.bsum);
+    k_scan_local<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, b.cursor);
+    k_scan1<<<1, 1024, 0, p->stream>>>((int)nb, b.bsum, b.cursor, b.occ);
     k_scan_add<<<(unsigned)std::min<int64_t>((nkeys + 255) / 256, 152 * 16), 256, 0, p->stream>>>(
         nkeys, b.hist, b.bsum, b.cursor, (unsigned)nb);
     timing_end(p, slot);
@@ -317,7 +329,7 @@ sl_status launch_sort_into(sl_plan *p, const SortBufs &b, const double *theta, c
     if ((st = cuda_check(cudaGetLastError(), "k_scatter_agg launch")) != SL_OK) return st;
     if (with_chunks) {
         k_tile_chunks<<<(p->ntiles + 255) / 256, 256, 0, p->stream>>>(p->ntiles, ncell, b.hist, b.chunk_off);
-        k_scan1<<<1, 1024, 0, p->stream>>>(p->ntiles, b.chunk_off);
+        k_scan1<<<1, 1024, 0, p->stream>>>(p->ntiles, b.chunk_off, nullptr, nullptr);
         st = cuda_check(cudaGetLastError(), "k_tile_chunks launch");
     }
     return st;

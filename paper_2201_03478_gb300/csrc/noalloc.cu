@@ -83,11 +83,12 @@ extern "C" sl_status interp_tod_noalloc(sl_plan *p, const void *maps, const doub
     b.hist = b.perm + kNoAllocMaxSamples;                  // cleared by the sort before use
     b.cursor = b.hist + (kNoAllocMaxTiles + 1);
     b.bsum = b.cursor + kNoAllocMaxTiles;
+    b.occ = nullptr;                                       // no count of occupied tiles
     const int rec64 = plan_wide(p->precision);
     // FP32, TF32X3 and DF64 plans interpolate tile by tile from shared memory and need
     // the per-tile work list; FP64 plans gather per sample and do not.
     const int chunks = p->precision != SL_FP64;
     b.chunk_off = chunks ? b.bsum + kBsumWords : nullptr;
     if ((st = launch_sort_into(p, b, theta, phi, psi, n, 0, rec64, chunks)) != SL_OK) return st;
-    return launch_interp(p, b, 0, maps, psi, n, tod);
+    return launch_interp(p, b, 0, maps, psi, n, n, tod);
 }

@@ -155,6 +155,7 @@ static sl_status alloc_sort_tables(sl_plan *p) {
     sl_status st = dalloc_t(p, &p->sort.hist, (size_t)p->nkeys + 1, "cell histogram");
     if (st == SL_OK) st = dalloc_t(p, &p->sort.cursor, (size_t)p->nkeys, "cell cursor");
     if (st == SL_OK) st = dalloc_t(p, &p->sort.bsum, (size_t)sort_nbsum(p->nkeys) + 2, "scan block sums");
+    if (st == SL_OK) p->sort.occ = p->sort.bsum + sort_nbsum(p->nkeys) + 1;
     if (st == SL_OK) st = dalloc_t(p, &p->sort.chunk_off, (size_t)p->ntiles + 1, "tile chunks");
     return st;
 }
@@ -164,7 +165,7 @@ static void free_sort_tables(sl_plan *p) {
     dfree(p->sort.cursor);
     dfree(p->sort.bsum);
     dfree(p->sort.chunk_off);
-    p->sort.hist = p->sort.cursor = p->sort.bsum = p->sort.chunk_off = nullptr;
+    p->sort.hist = p->sort.cursor = p->sort.bsum = p->sort.chunk_off = p->sort.occ = nullptr;
     p->bytes_held -= (int64_t)sizeof(unsigned) * ((p->nkeys + 1) + p->nkeys + (sort_nbsum(p->nkeys) + 2) +
                                                   (p->ntiles + 1));
 }
@@ -296,6 +297,7 @@ void plan_destroy(sl_plan *p) {
     dfree(p->d_ring_fix);
     dfree(p->d_wden);
     dfree(p->d_lut);
+    dfree(p->d_phase_tab);
     dfree(p->d_seed);
     dfree(p->d_seed_e);
     dfree(p->d_tab64);
@@ -555,6 +557,18 @@ sl_status sidelobe_plan_create(sl_plan **out, const sl_plan_desc *d) {
                               cudaMemcpyHostToDevice), "upload"));
     TRY(cuda_check(cudaMemcpy(p->d_offs64, offs64.data(), offs64.size() * sizeof(double), cudaMemcpyHostToDevice), "upload"));
     TRY(cuda_check(cudaMemcpy(p->d_rowtab32, rowtab32.data(), rowtab32.size() * sizeof(float), cudaMemcpyHostToDevice), "upload"));
+    {
+        std::vector<longlong2> pt(256);
+        for (int q = 0; q < 256; ++q) {
+            const long double a = 2.0L * 3.14159265358979323846264338327950288L * q / 256;
+            pt[(size_t)q].x = llroundl(ldexpl(cosl(a), 62));
+            pt[(size_t)q].y = llroundl(ldexpl(sinl(a), 62));
+        }
+        TRY(dalloc_t(p, &p->d_phase_tab, pt.size(), "phase table"));
+        TRY(cuda_check(cudaMemcpy(p->d_phase_tab, pt.data(), pt.size() * sizeof(longlong2), cudaMemcpyHostToDevice),
+                       "upload"));
+        p->geom.phase_tab = p->d_phase_tab;
+    }
     p->geom.ring_ext = p->d_ring_ext;
     p->geom.ring_fix = p->d_ring_fix;
     p->geom.wden = p->d_wden;
@@ -655,6 +669,19 @@ static sl_status check_ptg(const double *theta, const double *phi, const double 
     return SL_OK;
 }
 
+// The sort and interpolation of n samples of a TOD of n_total (the kernel is chosen by
+// the whole TOD, so that pieces of it get the same values).
+static sl_status interp_part(sl_plan *p, const void *maps, const double *theta, const double *phi, const double *psi,
+                             int64_t n, int64_t n_total, double *tod) {
+    sl_status st;
+    if ((st = ensure_sort_capacity(p, n)) != SL_OK) return st;
+    SortBufs b = p->sort;
+    const int chunks = interp_needs_chunks(p, n_total);
+    if (!chunks) b.chunk_off = nullptr;
+    if ((st = launch_sort_into(p, b, theta, phi, psi, n, 1, plan_wide(p->precision), chunks)) != SL_OK) return st;
+    return launch_interp(p, b, 1, maps, psi, n, n_total, tod);
+}
+
 sl_status interp_tod(sl_plan *p, const void *maps, const double *theta, const double *phi,
                      const double *psi, int64_t n, double *tod) {
     sl_status st = enter(p);
@@ -662,14 +689,7 @@ sl_status interp_tod(sl_plan *p, const void *maps, const double *theta, const do
     if ((st = check_ptg(theta, phi, psi, n, tod, "interp_tod")) != SL_OK) return st;
     if (!maps) return set_error(SL_ERR_ARG, "interp_tod: maps is NULL");
     if (n == 0) return SL_OK;
-    if ((st = ensure_sort_capacity(p, n)) != SL_OK) return st;
-    const int rec64 = plan_wide(p->precision);
-    // FP32 and DF64 plans interpolate tile by tile from shared memory (needs the work items)
-    SortBufs b = p->sort;
-    const int chunks = p->precision != SL_FP64;
-    if (!chunks) b.chunk_off = nullptr;
-    if ((st = launch_sort_into(p, b, theta, phi, psi, n, 1, rec64, chunks)) != SL_OK) return st;
-    return launch_interp(p, b, 1, maps, psi, n, tod);
+    return interp_part(p, maps, theta, phi, psi, n, n, tod);
 }
 
 sl_status convolve_tod(sl_plan *p, const double *sky, const double *beam, void *maps, const double *theta,
@@ -684,7 +704,7 @@ sl_status convolve_tod(sl_plan *p, const double *sky, const double *beam, void *
     if ((st = ensure_side_stream(p)) != SL_OK) return st;
     const int rec64 = plan_wide(p->precision);
     SortBufs b = p->sort;
-    const int chunks = p->precision != SL_FP64;
+    const int chunks = interp_needs_chunks(p, n);
     if (!chunks) b.chunk_off = nullptr;
     // fork point: everything queued on the plan's stream before the call
     if ((st = cuda_check(cudaEventRecord(p->side_fork, p->stream), "fork")) != SL_OK) return st;
@@ -698,7 +718,7 @@ sl_status convolve_tod(sl_plan *p, const double *sky, const double *beam, void *
     if ((st = launch_lcontract(p, sky, beam)) != SL_OK) return st;
     if ((st = launch_ringfft_synth(p, maps)) != SL_OK) return st;
     if ((st = cuda_check(cudaStreamWaitEvent(p->stream, p->side_join, 0), "join")) != SL_OK) return st;
-    return launch_interp(p, b, 1, maps, psi, n, tod);
+    return launch_interp(p, b, 1, maps, psi, n, n, tod);
 }
 
 // ---- end to end from host buffers
@@ -770,7 +790,8 @@ static sl_status host_pipeline(sl_plan *p, const double *sky, const double *beam
     for (int c = 0; c < np && st == SL_OK; ++c) {
         const int64_t a = n * c / np, b = n * (c + 1) / np;
         st = cuda_check(cudaStreamWaitEvent(p->stream, p->h_arrived[c], 0), "piece wait");
-        if (st == SL_OK && b > a) st = interp_tod(p, p->d_hmaps, d_th + a, d_ph + a, d_ps + a, b - a, p->d_htod + a);
+        if (st == SL_OK && b > a)
+            st = interp_part(p, p->d_hmaps, d_th + a, d_ph + a, d_ps + a, b - a, n, p->d_htod + a);
         if (st == SL_OK) st = cuda_check(cudaEventRecord(p->h_done[c], p->stream), "piece done");
         if (st == SL_OK) st = cuda_check(cudaStreamWaitEvent(p->down, p->h_done[c], 0), "download wait");
         if (st == SL_OK && b > a)
@@ -1190,7 +1211,7 @@ sl_status interp_tod_psi(sl_plan *p, const void *cube_psi, int npsi, const doubl
 
 unsigned sl_debug_check_status(void) {
     // every unit's word is read (and cleared); the first nonzero one is reported
-    const unsigned w[6] = {chk_sort(), chk_interp(), chk_interp_df(), chk_psigrid(), chk_orbital(), chk_fft()};
+    const unsigned w[7] = {chk_sort(), chk_interp(), chk_interp_df(), chk_interp_fx(), chk_psigrid(), chk_orbital(), chk_fft()};
     for (unsigned v : w)
         if (v) return v;
     return 0u;

@@ -60,6 +60,7 @@ struct InterpGeom {
     const double *offs64;         // [(R+1) * p]: theta(i0+a) - theta(i0), i0 = i - p/2 + 1, per base row i
     const float *rowtab32;        // [(R+1) * 2p]: the same offsets, then wden, in float
     const float2 *rowtab_df;      // [(R+1) * 2p]: the same, as double-float (hi, lo)
+    const longlong2 *phase_tab;   // [256]: (cos, sin)(2 pi i / 256) 2^62
 };
 
 // Bounds-checked builds (-DSL_CHECKED, the variant _build.build(checked=True) makes):
@@ -91,6 +92,7 @@ __device__ __forceinline__ bool sl_guard(bool ok, unsigned site) {
 unsigned chk_sort();
 unsigned chk_interp();
 unsigned chk_interp_df();
+unsigned chk_interp_fx();
 unsigned chk_psigrid();
 unsigned chk_orbital();
 unsigned chk_fft();
@@ -223,6 +225,7 @@ struct SortBufs {
     unsigned *cursor;     // [nkeys]
     unsigned *bsum;       // [nkeys / 4096 + 2]
     unsigned *chunk_off;  // [ntiles + 1]
+    unsigned *occ;        // keys that hold samples (in bsum's last entry; written by the sort)
 };
 
 // Rescaled l-recurrence coefficients per (k, m, l), stored at
@@ -260,6 +263,7 @@ struct sl_plan {
     float *d_rowtab32 = nullptr;
     float2 *d_rowtab_df = nullptr;
     int *d_lut = nullptr;
+    longlong2 *d_phase_tab = nullptr;
     int nlut = 0;
     sl::InterpGeom geom;
 
@@ -303,7 +307,7 @@ struct sl_plan {
     // pointing sort (fine cell keys; per-sample scratch grown on demand)
     int ntiles = 0;
     int64_t nkeys = 0;
-    sl::SortBufs sort = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    sl::SortBufs sort = {};
     int64_t sort_cap = 0;
 
     int64_t bytes_held = 0;
@@ -445,8 +449,15 @@ sl_status launch_sort_into(sl_plan *p, const SortBufs &b, const double *theta, c
 TiledArgs fine_tiled_args(const sl_plan *p, const SortBufs &b, const void *maps, double *tod);
 sl_status launch_interp_f32_cells(cudaStream_t stream, int device, const TiledArgs *dets, int nd, int tc, int P,
                                   int kmax_max, unsigned *work, int *err);
+// n of the n_total samples of the call's TOD: the kernel is chosen by n_total.
 sl_status launch_interp(sl_plan *p, const SortBufs &b, int fine, const void *maps, const double *psi, int64_t n,
-                        double *tod);
+                        int64_t n_total, double *tod);
+// whether that interpolation of a sort by cell reads the sort's work items (chunk_off)
+int interp_needs_chunks(const sl_plan *p, int64_t n_total);
+// FP64 and DF64 plans over a sort by cell: the sums on the tensor cores (k_interp_fx.cu),
+// where interp_uses_fx
+bool interp_uses_fx(const sl_plan *p, int64_t n_total);
+sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n, double *tod);
 size_t interp_f32_tiled_smem(const sl_plan *p);
 // Dynamic shared memory of the two tile-staged kernels for tile width tc.
 size_t interp_f32_tiled_smem_tc(const sl_plan *p, int tc);
