@@ -223,14 +223,15 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
     # 11 flops (3 recurrence + 2 complex x real MACs) per visited (ring, m, k, sign, l)
     fl_lc = 11.0 * lsteps
     suffix = {"fp64": "f64", "fp32": "f32", "df64": "df", "tf32x3": "f32"}[prec]
-    lc_name = "lcontract_mma" if prec == "tf32x3" else "lcontract_" + suffix
+    lc_name = {"tf32x3": "lcontract_mma", "fp64": "lcontract_fx"}.get(prec, "lcontract_" + suffix)
     meas = {"fp64": alu.get("fp64"), "fp32": alu.get("fp32")}
     kernels = [
         (lc_name,
-         {"fp64": fl_lc, "fp32": fl_lc, "df64": DF_LC_INST_PER_STEP * lsteps,
+         # FP64: digit products executed, 60 m16n8k8 per 32 recurrences and 8 l
+         {"fp64": 60 * 2.0 * 16 * 8 * 8 / 256 * lsteps, "fp32": fl_lc, "df64": DF_LC_INST_PER_STEP * lsteps,
           # tensor work executed: 3 TF32 products x 2 flops x 16 columns (4 used, one sky)
           "tf32x3": 3 * 2.0 * 16 * lsteps}[prec],
-         {"fp64": "fp64", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "tf32"}[prec]),
+         {"fp64": "fp16", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "tf32"}[prec]),
         ("interp_" + suffix, float(n) * df_interp_inst(K) if prec == "df64" else fl_in,
          {"fp64": "fp64", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "fp32"}[prec]),
         # FP64 and DF64 plans: 27 digit products per 8 orders, m16n8k16, 8 samples a group

@@ -89,6 +89,12 @@ __device__ __forceinline__ void mma_f16(float &c0, float &c1, float &c2, float &
             : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// c += A B on 16 x 8 x 8 FP16 fragments
+__device__ __forceinline__ void mma_f16_k8(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(b));
+}
+
 // xh (digits 0..2) and xl (digits 3..5) of a Q62 value
 __device__ __forceinline__ void fx_split(long long x, int &h, int &l) {
     constexpr int kBias27 = (1 << 26) + (1 << 17) + (1 << 8);       // 256 in each of three digits

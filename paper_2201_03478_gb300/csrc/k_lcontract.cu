@@ -27,8 +27,7 @@
 // l at which the value is significant; the evanescent part before it (about
 // 28% of the (ring, m, l) volume at lmax = 1024) is not run at all.
 //
-// FP64 plans: one thread per (north ring, sign of k): per l, 2 FP64 operations
-// for the recurrence and 4 for the two complex x real sums.  FP32 plans: eight
+// FP64 plans: k_lcontract_fx.cu (fixed point and tensor cores).  FP32 plans: eight
 // ring pairs per thread of one sign, two at a time in the lanes of packed FP32x2
 // instructions (k_lcontract_f32); the recurrence in the
 // difference form  D_{l+1} = (c'_l - a'_l y) y_l + D_l,  y_{l+1} = y_l + D_{l+1}
@@ -39,7 +38,7 @@
 // and the sums in double-float arithmetic (df.cuh): per l, two double-float
 // products and two sums for the recurrence and four double-float
 // multiply-accumulates, all on the FP32 pipes.
-// FP64 and DF64: the CTA stages the coefficients of a chunk of l in shared
+// DF64: the CTA stages the coefficients of a chunk of l in shared
 // memory and a thread steps only from its own start l.  FP32: each warp stages
 // its own coefficients, 32 l at a time, and steps from its earliest start
 // (recurrences not yet started hold an exact zero state).
@@ -47,7 +46,7 @@
 #include <vector>
 
 #include "df.cuh"
-#include "sl_internal.cuh"
+#include "lcontract.cuh"
 
 namespace sl {
 
@@ -55,70 +54,7 @@ constexpr int kNT = 256;          // threads per CTA
 constexpr int kHalf = kNT / 2;    // threads per sign
 constexpr int kNT32 = 128;        // threads per CTA of the FP32 contraction: 64 per sign of k,
 constexpr int kHalf32 = kNT32 / 2;   // 2, 4 or 8 ring pairs each (lcontract_f32_ppt)
-constexpr int kLC64 = 64;         // l values staged per chunk (FP64)
-
-struct __align__(16) Coef64 {
-    double a, nb, pb, unused;     // a', -b', +b'
-};
-struct __align__(16) Acc64 {
-    double2 ap, sam, am, sap;     // +k uses (ap, sam), -k uses (am, sap)
-};
-
-struct LcArgs {
-    int L, K, ncomp, R, npairs, nchunk, ppt;  // ppt: ring pairs per thread
-    int64_t nalm;
-    const double2 *sky, *beam;       // FP64 inputs
-    const float2 *sky32, *beam32;    // FP32 copies (FP32 plans)
-    const double *xr;
-    const float *y32;
-    const int *ls;
-    const double2 *st64;
-    const float2 *st32;
-    const RTab64 *tab64;
-    const RTab32 *tab32;
-    void *G;
-};
-
-// Block b -> (m, k, ring chunk pc).
-__device__ __forceinline__ void block_mk_of(const LcArgs &a, int b, int &m, int &k, int &pc) {
-    pc = b % a.nchunk;
-    b /= a.nchunk;
-    k = b % (a.K + 1);
-    m = b / (a.K + 1);
-}
-__device__ __forceinline__ void block_mk(const LcArgs &a, int &m, int &k, int &pc) { block_mk_of(a, blockIdx.x, m, k, pc); }
-
-__device__ __forceinline__ int64_t start_index(const LcArgs &a, int k, int m, int neg, int pair) {
-    return (((int64_t)k * (a.L + 1) + m) * 2 + neg) * a.npairs + pair;
-}
-
-// Writes the two sums of one recurrence.  neg = 0 (+k): acc1 -> (north, +m),
-// acc2 -> (south, -m); neg = 1 (-k): acc1 -> (north, -m), acc2 -> (south, +m).
-template <typename C>
-__device__ __forceinline__ void write_two(const LcArgs &a, int m, int k, int pair, int neg, C acc1, C acc2) {
-    C *G = reinterpret_cast<C *>(a.G);
-    const int rn = pair, rs = a.R - 1 - pair;
-    // rows (k, L + m) and (k, L - m) of G
-    C *gp = G + ((int64_t)k * (2 * a.L + 1) + a.L + m) * a.R;
-    C *gm = G + ((int64_t)k * (2 * a.L + 1) + a.L - m) * a.R;
-    const bool modd = m & 1, kodd = k & 1;
-    if (!neg) {
-        gp[rn] = acc1;
-        if (m > 0 && rs != rn) {
-            if (modd != kodd) { acc2.x = -acc2.x; acc2.y = -acc2.y; }
-            gm[rs] = acc2;
-        }
-    } else {
-        if (m > 0) {
-            if (kodd) { acc1.x = -acc1.x; acc1.y = -acc1.y; }
-            gm[rn] = acc1;
-        }
-        if (rs != rn) {
-            if (modd) { acc2.x = -acc2.x; acc2.y = -acc2.y; }
-            gp[rs] = acc2;
-        }
-    }
-}
+constexpr int kLC64 = 64;         // l values staged per chunk (DF64)
 
 // Smallest start l over the CTA (L + 1 when no thread has work).
 __device__ __forceinline__ int block_min(int v) {
@@ -128,75 +64,6 @@ __device__ __forceinline__ int block_min(int v) {
     atomicMin(&s_min, v);
     __syncthreads();
     return s_min;
-}
-
-// ------------------------------------------------------------------ FP64
-__global__ void __launch_bounds__(kNT) k_lcontract_f64(const LcArgs a) {
-    __shared__ Coef64 rc[kLC64];
-    __shared__ Acc64 ac[kLC64];
-    int m, k, pc;
-    block_mk(a, m, k, pc);
-    const int neg = threadIdx.x >= kHalf;
-    const int pair = pc * kHalf + (threadIdx.x & (kHalf - 1));
-    const bool active = pair < a.npairs;
-    const int64_t moff = (int64_t)m * (2 * a.L + 1 - m) / 2;
-    const RTab64 *tab = a.tab64 + (int64_t)k * a.nalm + moff;
-
-    double x = 0.0, y = 0.0, yo = 0.0;
-    int ls = a.L + 1;
-    if (active) {
-        const int64_t si = start_index(a, k, m, neg, pair);
-        ls = a.ls[si];
-        const double2 s = a.st64[si];
-        yo = s.x;
-        y = s.y;
-        x = a.xr[pair];
-    }
-    double2 acc1 = {0, 0}, acc2 = {0, 0};
-    const int lstart = block_min(ls);
-    // coefficient slots of this thread's sign
-    const int bofs = neg ? 2 : 1;     // index of -b' (for +k) or +b' (for -k) in Coef64
-    const int cofs = neg ? 2 : 0;     // first double2 of (ap, sam) or (am, sap) in Acc64
-    for (int c0 = lstart; c0 <= a.L; c0 += kLC64) {
-        const int nc = min(kLC64, a.L - c0 + 1);
-        __syncthreads();
-        for (int i = threadIdx.x; i < nc; i += kNT) {
-            const int l = c0 + i;
-            const RTab64 t = tab[l];
-            rc[i] = Coef64{t.a, -t.b, t.b, 0.0};
-            double2 ap = {0.0, 0.0}, am = {0.0, 0.0};
-            for (int X = 0; X < a.ncomp; ++X) {
-                double2 s = a.sky[X * a.nalm + moff + l];
-                if (m == 0) s.y = 0.0;
-                double2 b = a.beam[((int64_t)X * (a.K + 1) + k) * (a.L + 1) + l];
-                if (k == 0) b.y = 0.0;
-                ap.x += s.x * b.x + s.y * b.y;      // s conj(b)
-                ap.y += s.y * b.x - s.x * b.y;
-                am.x += s.x * b.x - s.y * b.y;      // conj(s) conj(b)
-                am.y -= s.y * b.x + s.x * b.y;
-            }
-            const double c = t.c, sc = (l & 1) ? -c : c;
-            ac[i] = Acc64{make_double2(c * ap.x, c * ap.y), make_double2(sc * am.x, sc * am.y),
-                          make_double2(c * am.x, c * am.y), make_double2(sc * ap.x, sc * ap.y)};
-        }
-        __syncthreads();
-        const int i0 = max(0, ls - c0);
-        const double *rcd = reinterpret_cast<const double *>(rc);
-        const double2 *acd = reinterpret_cast<const double2 *>(ac);
-#pragma unroll 4
-        for (int i = i0; i < nc; ++i) {
-            const double ra = rcd[4 * i], rb = rcd[4 * i + bofs];
-            const double2 c1 = acd[4 * i + cofs], c2 = acd[4 * i + cofs + 1];
-            acc1.x = fma(c1.x, y, acc1.x);
-            acc1.y = fma(c1.y, y, acc1.y);
-            acc2.x = fma(c2.x, y, acc2.x);
-            acc2.y = fma(c2.y, y, acc2.y);
-            const double yn = fma(fma(ra, x, rb), y, -yo);
-            yo = y;
-            y = yn;
-        }
-    }
-    if (active) write_two<double2>(a, m, k, pair, neg, acc1, acc2);
 }
 
 // ------------------------------------------------------------------ FP32
@@ -672,15 +539,13 @@ sl_status launch_lcontract(sl_plan *p, const double *sky, const double *beam) {
         return launch_lcontract_mma(p, 1, sky, beam, p->d_sky32, (float2 *)p->d_G, p->d_err);
     LcArgs a;
     make_lcargs(p, sky, beam, a);
+    if (p->precision == SL_FP64) return launch_lcontract_fx(p, a);
     const int64_t nblk = (int64_t)(p->L + 1) * (p->K + 1) * a.nchunk;
     if (nblk > 0x7fffffff) return set_error(SL_ERR_UNSUPPORTED, "grid too large");
     int slot;
     if (p->precision == SL_DF64) {
         slot = timing_begin(p, "lcontract_df");
         k_lcontract_df<<<(unsigned)nblk, kNT, 0, p->stream>>>(a);
-    } else if (p->precision == SL_FP64) {
-        slot = timing_begin(p, "lcontract_f64");
-        k_lcontract_f64<<<(unsigned)nblk, kNT, 0, p->stream>>>(a);
     } else {
         sl_status st = launch_to_f32(p, p->stream, sky, beam);
         if (st != SL_OK) return st;

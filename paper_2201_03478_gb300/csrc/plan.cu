@@ -300,6 +300,7 @@ void plan_destroy(sl_plan *p) {
     dfree(p->d_phase_tab);
     dfree(p->d_seed);
     dfree(p->d_seed_e);
+    dfree(p->d_lc_counter);
     dfree(p->d_tab64);
     dfree(p->d_tab32);
     if (p->d_ls_adj && p->d_ls_adj != p->d_ls) dfree(p->d_ls_adj);
@@ -612,6 +613,7 @@ sl_status sidelobe_plan_create(sl_plan **out, const sl_plan_desc *d) {
         TRY(dalloc(p, &p->d_G, p->G_bytes, "spin-Legendre scratch G"));
     }
     TRY(alloc_sort_tables(p));
+    if (plan_wide(p->precision)) TRY(dalloc_t(p, &p->d_lc_counter, 1, "contraction counter"));
     if (plan_fp32(p->precision)) {
         // [0]: device flag of the bounded waits (FP32 interpolation, tensor-core contraction);
         // [1]: work counter of the FP32 interpolation

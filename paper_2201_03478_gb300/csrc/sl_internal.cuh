@@ -279,6 +279,7 @@ struct sl_plan {
     double2 *d_st64 = nullptr;
     float2 *d_st32 = nullptr;
     int64_t lsteps = 0;               // recurrence steps per synth call
+    unsigned *d_lc_counter = nullptr;   // unit counter of the fixed-point contraction (FP64, DF64 plans)
     // FP64 start states of the adjoint contraction (alias the above in FP64 plans)
     int *d_ls_adj = nullptr;
     double2 *d_st64_adj = nullptr;
