@@ -38,8 +38,8 @@
 // plain FP64 loop (the sums then overflow or turn NaN where that form does).
 #include <algorithm>
 
-#include "fxdigits.cuh"
 #include "lcontract.cuh"
+#include "lfrec.cuh"
 
 namespace sl {
 
@@ -84,49 +84,12 @@ __device__ __forceinline__ void lf_columns(const LcArgs &a, int64_t moff, int m,
     v[3] = -sc * (r + t);
 }
 
-// One fixed-point step Y_{l+1} = t Y_l - Y_{l-1}, t = a' x - b', |t| < 4, |Y| < 2^60.  Words
-// are split where the products need no shift: a' = Ah 2^-27 + Al 2^-58, x = xh 2^-31 + xl 2^-62,
-// t = th 2^-29 + tl 2^-58 and Y = Yh 2^29 + Yl with 29-bit tl, Yl >= 0.  The two low x high
-// products share a 64-bit sum whose carry into the units is rounded; tl Yl (a quarter unit on
-// average, like the half) is in the rounding constant.
-struct LfRec {
-    long long Y, Yo;
-    int xh, xl;
-    __device__ __forceinline__ void step(const int4 c) {
-        const long long B = (long long)(((unsigned long long)(unsigned)c.w << 32) | (unsigned)c.z);
-        const long long mt = (long long)c.x * xl + ((long long)c.y * xh + (1ll << 30));
-        const long long t = (long long)c.x * xh + ((mt >> 31) + B);
-        const int th = (int)(t >> 29), tl = (int)t & 0x1fffffff;
-        const int Yh = (int)(Y >> 29), Yl = (int)Y & 0x1fffffff;
-        const long long m = (long long)th * Yl + ((long long)tl * Yh + 3 * (1ll << 27));
-        const long long Yn = (long long)th * Yh + ((m >> 29) - Yo);
-        Yo = Y;
-        Y = Yn;
-    }
-};
-
-// Seven digits of two values Y 2^-60 in (-1, 1): fields of Y + bias at bits 52, 43, .., 7 and the
-// last seven bits; a field that lies within a 16-bit half is cut from both values' halves at once.
-__device__ __forceinline__ uint32_t lf_digit(uint32_t u, uint32_t mask) {
-    u = (u & mask) | 0x64006400u;
-    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&u), __halves2half2(__ushort_as_half(0x6500), __ushort_as_half(0x6500)));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
 __device__ __forceinline__ void lf_store(LfWarp &W, int pr, int lane, long long v0, long long v1) {
-    constexpr unsigned long long kBias = (1ull << 60) + (1ull << 51) + (1ull << 42) + (1ull << 33) + (1ull << 24) +
-                                         (1ull << 15) + (1ull << 6);
-    const unsigned long long a = (unsigned long long)v0 + kBias, b = (unsigned long long)v1 + kBias;
-    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
-    const uint32_t w3 = __byte_perm(ah, bh, 0x7632), w2 = __byte_perm(ah, bh, 0x5410);
-    const uint32_t w1 = __byte_perm(al, bl, 0x7632), w0 = __byte_perm(al, bl, 0x5410);
-    uint32_t *d = &W.yd[0][pr][lf_slot(pr, lane)];
-    d[0 * 128] = lf_digit(w3 >> 4, 0x03ff03ffu);
-    d[1 * 128] = lf_digit(__byte_perm(ah >> 11, bh >> 11, 0x5410), 0x01ff01ffu);
-    d[2 * 128] = lf_digit(w2 >> 2, 0x01ff01ffu);
-    d[3 * 128] = lf_digit(__byte_perm(__funnelshift_r(al, ah, 25), __funnelshift_r(bl, bh, 25), 0x5410), 0x01ff01ffu);
-    d[4 * 128] = lf_digit(w1, 0x01ff01ffu);
-    d[5 * 128] = lf_digit(w0 >> 7, 0x01ff01ffu);
-    d[6 * 128] = lf_digit(w0 << 2, 0x01fc01fcu);
+    uint32_t d[7];
+    lf_digits(v0, v1, d);
+    uint32_t *o = &W.yd[0][pr][lf_slot(pr, lane)];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) o[128 * j] = d[j];
 }
 
 // The plain FP64 loop of one ring , out of line (rare).
@@ -164,11 +127,7 @@ __device__ __forceinline__ void lf_batch(const LcArgs &a, LfWarp &W, int grp, bo
     double y = 0.0, yo = 0.0;
     LfRec r;
     r.Y = r.Yo = 0;
-    {   // x 2^62 as xh 2^31 + xl, |xl| <= 2^30
-        const long long X = min(fx_from_double(x, 1023), (1ll << 61) - 1) * 2;
-        r.xh = (int)((X + (1ll << 30)) >> 31);
-        r.xl = (int)(X - ((long long)r.xh << 31));
-    }
+    lf_set_x(r, x);
     const longlong2 st = W.state[grp][lane];
     const double so = __longlong_as_double(st.x), sv = __longlong_as_double(st.y);
     if (fixed) {
@@ -195,8 +154,8 @@ __device__ __forceinline__ void lf_batch(const LcArgs &a, LfWarp &W, int grp, bo
         grown |= ls < lk && fmax(fabs(y), fabs(yo)) >= big;
         if (!fixed && !(steep >> (8 * ks)) && __all_sync(0xffffffffu, grown || ls > a.L)) {
             fixed = true;
-            r.Y = (fx_from_double(y, U + 1022) + 2) >> 2;
-            r.Yo = (fx_from_double(yo, U + 1022) + 2) >> 2;
+            r.Y = lf_from_double(y, U);
+            r.Yo = lf_from_double(yo, U);
         }
         // two l per round, rolled: unrolled, the two forms do not fit the instruction cache
         if (fixed) {
@@ -320,10 +279,9 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
             x0 = x;
         }
     }
-    // |y| < 2^U for every ring and l: |d| < 1 (but for l = 0), c >= cmin >= 2^(ex - 1023)
     double cmin = tab[a.L].c;
     if (a.L > max(m, k)) cmin = fmin(cmin, tab[a.L - 1].c);
-    const int U = max(1, 1023 - ((__double2hiint(cmin) >> 20) & 0x7ff));
+    const int U = lf_bound(cmin);
     const int lfirst0 = __reduce_min_sync(0xffffffffu, W.ls[0][lane] >> 1);
     bool fixed0 = false, fixed1 = false;
 
@@ -343,12 +301,9 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
                 lf_columns(a, moff, m, k, l, t.c, v[h]);
             }
             W.cd[i] = make_double2(t.a, -t.b);
-            // a' + |b'| >= 4: the batch's FP64 steps cover it (a' falls with l)
-            const bool big = t.a + fabs(t.b) >= 4.0;
+            bool big;                   // the batch's FP64 steps cover these (a' falls with l)
+            W.ci[i] = lf_coef(t.a, t.b, big);
             steep |= (uint64_t)__ballot_sync(0xffffffffu, big) << (32 * h);
-            const long long A = big ? 0 : fx_from_double(t.a, 1026), B = big ? 0 : fx_from_double(-t.b, 1026);  // 2^58
-            const int Ah = (int)((A + (1ll << 30)) >> 31);
-            W.ci[i] = make_int4(Ah, (int)(A - ((long long)Ah << 31)), (int)B, (int)(B >> 32));
 #pragma unroll
             for (int c = 0; c < 4; ++c) mx = max(mx, (uint32_t)__double2hiint(v[h][c]) & 0x7fffffffu);
         }

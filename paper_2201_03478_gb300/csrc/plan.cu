@@ -613,7 +613,7 @@ sl_status sidelobe_plan_create(sl_plan **out, const sl_plan_desc *d) {
         TRY(dalloc(p, &p->d_G, p->G_bytes, "spin-Legendre scratch G"));
     }
     TRY(alloc_sort_tables(p));
-    if (plan_wide(p->precision)) TRY(dalloc_t(p, &p->d_lc_counter, 1, "contraction counter"));
+    TRY(dalloc_t(p, &p->d_lc_counter, 1, "contraction counter"));
     if (plan_fp32(p->precision)) {
         // [0]: device flag of the bounded waits (FP32 interpolation, tensor-core contraction);
         // [1]: work counter of the FP32 interpolation

@@ -279,7 +279,7 @@ struct sl_plan {
     double2 *d_st64 = nullptr;
     float2 *d_st32 = nullptr;
     int64_t lsteps = 0;               // recurrence steps per synth call
-    unsigned *d_lc_counter = nullptr;   // unit counter of the fixed-point contraction (FP64, DF64 plans)
+    unsigned *d_lc_counter = nullptr;   // unit counter of the fixed-point contraction and its transpose
     // FP64 start states of the adjoint contraction (alias the above in FP64 plans)
     int *d_ls_adj = nullptr;
     double2 *d_st64_adj = nullptr;
@@ -477,6 +477,7 @@ sl_status launch_interp_adjoint(sl_plan *p, const SortBufs &b, int fine, const d
                                 int64_t n, double2 *fbar);
 sl_status launch_ringdft_adjoint(sl_plan *p, const double2 *fbar);
 sl_status launch_lcontract_adjoint(sl_plan *p);
+sl_status launch_lcontract_adj_fx(sl_plan *p);   // over a zeroed Abar (k_adjoint_fx.cu)
 sl_status launch_grad(sl_plan *p, const double *sky, const double *beam, double *sky_grad,
                       double *beam_grad, int accumulate);
 
