@@ -646,6 +646,9 @@ struct AdjArgs {
     const double *psi, *y;
     const StencilRec64 *rec;
     const unsigned *perm, *start, *chunk_off;
+    const unsigned *occ;       // with min_mean: k_interp_adj_fx runs instead if n >= min_mean *occ
+    float min_mean;
+    int64_t n;
     int ntiles, ncell;
     double2 *fbar;
 };
@@ -657,6 +660,7 @@ template <int P>
 __global__ void k_interp_adjoint(const AdjArgs A) {
     constexpr int NQ = P * P;               // stencil nodes
     const InterpGeom &g = A.g;
+    if (A.occ && (float)A.n >= A.min_mean * (float)*A.occ) return;
     const int K1 = g.K + 1;
     const int TC = g.tile_cols;
     const int tw = TC + P - 1;              // smem tile columns
@@ -927,7 +931,14 @@ size_t interp_adjoint_smem_tc(const sl_plan *p, int tc) {
 
 sl_status launch_interp_adjoint(sl_plan *p, const SortBufs &b, int fine, const double *psi, const double *tod,
                                 int64_t n, double2 *fbar) {
-    if (p->precision == SL_DF64) return launch_interp_adjoint_df(p, b, fine, psi, tod, fbar);
+    float min_mean = 0.f;
+    const AdjRoute route = fine ? interp_adj_route(p, n, &min_mean) : AdjRoute::tiled;
+    const unsigned *occ = route == AdjRoute::by_occupancy ? b.occ : nullptr;
+    if (route != AdjRoute::tiled) {
+        const sl_status st = launch_interp_adj_fx(p, b, psi, tod, n, occ, min_mean, fbar);
+        if (st != SL_OK || route == AdjRoute::fx) return st;
+    }
+    if (p->precision == SL_DF64) return launch_interp_adjoint_df(p, b, fine, psi, tod, n, occ, min_mean, fbar);
     AdjArgs a;
     a.g = p->geom;
     a.psi = psi;
@@ -936,6 +947,9 @@ sl_status launch_interp_adjoint(sl_plan *p, const SortBufs &b, int fine, const d
     a.perm = b.perm;
     a.start = b.hist;
     a.chunk_off = b.chunk_off;
+    a.occ = occ;
+    a.min_mean = min_mean;
+    a.n = n;
     a.ntiles = p->ntiles;
     a.ncell = fine ? kTileRows * p->geom.tile_cols : 1;
     a.fbar = fbar;
@@ -961,7 +975,6 @@ sl_status launch_interp_adjoint(sl_plan *p, const SortBufs &b, int fine, const d
     int slot = timing_begin(p, "interp_adj");
     kern<<<(unsigned)(nsm * per_sm), 32 * nwarps, sm, p->stream>>>(a);
     timing_end(p, slot);
-    (void)n;
     return cuda_check(cudaGetLastError(), "k_interp_adjoint launch");
 }
 

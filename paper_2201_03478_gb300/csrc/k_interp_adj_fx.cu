@@ -1,0 +1,397 @@
+// k_interp_adj_fx.cu -- transpose of the interpolation (k_interp.cu: maps_bar_k(node) +=
+// w_node y eps_k e^{-ik psi}) in fixed point and on the tensor cores, at p = 4:
+//
+//   Fbar[q][c] = sum_s (y_s w_q(s)) E_c(s),   q: 16 nodes of the cell, c: (cos, -sin)(k psi_s)
+//
+// The FP64 form (k_interp_adjoint) was bound by the FP64 pipe: 2 p^2 (K + 1) multiply-adds a
+// sample at 1/64 of the FP32 rate.  Here both factors are
+// split into FP16 digits (fxdigits.cuh) and summed over 16 samples of a cell per mma.sync
+// m16n8k16, exactly; the 16 nodes of a 4 x 4 stencil are the 16 rows of the tile (as in
+// k_interp_fx, tcgen05's 128 rows would be mostly padding).
+//
+// One warp walks a stretch of the sorted samples in batches of 32:
+//   1. lane per sample: weights and phases in fixed point (fx_sincos; X_{k+1} = 2 cos psi X_k -
+//      X_{k-1}), y w_q relative to the largest |y| of the sample's run of equal cells, as
+//      digits to the warp's shared memory, [digit][node or real][sample];
+//   2. per 4 orders (their phases' digits made just before) and run: A = the run's columns
+//      (the others masked to zero), 27 digit products per 16 samples (order 0: E = 1, six),
+//      recombined and added to 64-bit sums in shared memory with an exponent per column.
+// The node of row q is kept at slot (column mod 4): when the run moves to a neighbouring cell
+// only the columns that leave the stencil are added to the cube (atomically), a quarter of the
+// values when the next cell is the next column.
+//
+// Measured (before -> after): 5e6 scanning samples at K = 16, 1024 x 2048 cells 7.62 -> 1.46 ms;
+// 2e7 uniform ones there 28.5 -> 15.9 ms (9.5 a cell); 1e7 at K = 4, 127 x 128 cells 5.21 -> 1.86 ms.
+// Bound by issue and the integer pipe (54% and 46% of their rates at 48 samples a cell, K = 16,
+// with 2.8 warps a scheduler): digits of 16 nodes and 2 K + 1 phases a sample, recombination a run.
+//
+// A sample with a non-finite y or psi, |y| outside 2^-959 .. 2^960, or weights out of the
+// fixed-point range is scattered in FP64 (adj_one).
+#include <algorithm>
+
+#include "fxdigits.cuh"
+#include "fxweights.cuh"
+#include "interp_f64.cuh"
+#include "mbar.cuh"
+#include "sl_internal.cuh"
+
+namespace sl {
+
+constexpr int kFaWarps = 4;
+constexpr int kFaRow = 20;         // words per row of 32 samples (padded: fragment rows in distinct banks)
+constexpr int kFaEmpty = -4096;    // exponent of sums that are all zero
+constexpr int kFaChunk = 512;      // longest stretch of a warp: keeps the 64-bit sums in range
+
+struct FaWarp {                    // one warp's shared memory; sums follow (fa_sums)
+    uint32_t a[6][16][kFaRow];     // digits of y w: [digit][4 row + column mod 4][sample pair]
+    uint32_t e[6][8][kFaRow];      // digits of the phases of 4 orders: [digit][2 order + part][sample pair]
+};
+// bytes per warp with the sums of order 0 (2 rows) and of blocks of 4 orders (2 rows x re, im)
+__host__ __device__ __forceinline__ size_t fa_warp_bytes(int nblk) {
+    return sizeof(FaWarp) + (size_t)(2 + 4 * nblk) * 32 * sizeof(long long);
+}
+
+struct FaArgs {
+    InterpGeom g;
+    const double *psi, *y;
+    const StencilRec64 *rec;
+    const unsigned *perm;
+    const unsigned *occ;           // with min_mean: run only if n >= min_mean *occ
+    float min_mean;
+    int64_t n;
+    int chunk;
+    double2 *fbar;
+};
+
+// Cube element of stencil row a's and column col's node (order 0) and whether odd orders flip.
+__device__ __forceinline__ int64_t fa_node(const InterpGeom &g, int row, int col, bool &flip) {
+    int ring = row;
+    flip = row < 0 || row >= g.R;
+    if (flip) {
+        ring = (row < 0) ? -1 - row : 2 * g.R - 1 - row;
+        col += g.nphi >> 1;
+    }
+    col = (col < 0) ? col + g.nphi : (col >= g.nphi ? col - g.nphi : col);
+    if (!SL_GUARD(ring >= 0 && ring < g.R && col >= 0 && col < g.nphi, 0x221u)) return 0;
+    return ((int64_t)ring * g.nphi + col) * (g.K + 1);
+}
+
+// One sample in FP64 (rare).
+__device__ __noinline__ void adj_one(const FaArgs &A, unsigned s) {
+    const InterpGeom &g = A.g;
+    const StencilRec64 r = A.rec[s];
+    const int i = (int)(r.cell >> 16) - 1, j = (int)(r.cell & 0xffffu);
+    double wt[4], wp[4], sp, cp;
+    weights64<4>(g, i, r.dth, r.fph, wt, wp);
+    sincos(A.psi[s], &sp, &cp);
+    const double y = A.y[s], c2 = 2.0 * cp;
+    for (int q = 0; q < 16; ++q) {
+        bool flip;
+        double2 *o = A.fbar + fa_node(g, i - 1 + q / 4, j - 1 + q % 4, flip);
+        const double w = wt[q / 4] * wp[q % 4];
+        double ck = 1.0, sk = 0.0, ckm = cp, skm = -sp;
+        for (int k = 0; k <= g.K; ++k) {
+            const double f = ((flip && (k & 1)) ? -w : w) * (k ? 2.0 * y : y);
+            atomicAdd(&o[k].x, f * ck);
+            atomicAdd(&o[k].y, -f * sk);
+            const double cn = fma(c2, ck, -ckm), sn = fma(c2, sk, -skm);
+            ckm = ck;
+            skm = sk;
+            ck = cn;
+            sk = sn;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid_constant__ FaArgs A) {
+    const InterpGeom &g = A.g;
+    if (A.occ && (float)A.n < A.min_mean * (float)*A.occ) return;   // few samples per cell: k_interp_adjoint
+    extern __shared__ __align__(16) unsigned char fa_smem[];
+    longlong2 *ptab = reinterpret_cast<longlong2 *>(fa_smem);
+    for (int q = threadIdx.x; q < 256; q += 32 * kFaWarps) ptab[q] = __ldg(g.phase_tab + q);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gr = lane >> 2, q4 = lane & 3;
+    const int nblk = (g.K + 3) >> 2;
+    FaWarp &W = *reinterpret_cast<FaWarp *>(fa_smem + 256 * sizeof(longlong2) + (size_t)warp * fa_warp_bytes(nblk));
+    // this lane's sums, times 2^(54 - exponent): order 0 of rows gr and gr + 8 (lanes q4 = 0), then
+    // per block b re and im of order 1 + 4 b + q4 of both rows
+    long long *sums = reinterpret_cast<long long *>(&W + 1) + lane;
+    const int64_t wfirst = ((int64_t)blockIdx.x * kFaWarps + warp) * A.chunk, wlast = min(A.n, wfirst + A.chunk);
+    if (wfirst >= wlast) return;
+    for (int v = 0; v < 2 + 4 * nblk; ++v) sums[32 * v] = 0;
+    int ecur = kFaEmpty;                            // exponent of this lane's column's sums
+    unsigned cur = 0xffffffffu;                     // the cell whose stencil the sums belong to
+
+    // adds the columns [c_lo, c_hi) (at most four, those of cell c) of block b (-1: order 0) to the cube
+    auto flush = [&](int b, unsigned c, int &e, int c_lo, int c_hi) {
+        const int i = (int)(c >> 16) - 1;
+        // this lane's rows both lie in slot gr & 3: the stencil column with that residue
+        const int col = c_lo + ((gr - c_lo) & 3);
+        if (col >= c_hi || e == kFaEmpty) return;
+        const double sc = __longlong_as_double((long long)(1023 + e - 54) << 52);
+        const int k = 1 + 4 * b + q4;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            bool flip;
+            double2 *o = A.fbar + fa_node(g, i - 1 + (gr >> 2) + 2 * h, col, flip);
+            if (b < 0) {
+                if (q4 == 0 && sums[32 * h]) atomicAdd(&o[0].x, (double)sums[32 * h] * sc);
+                sums[32 * h] = 0;
+            } else {
+                long long *v = sums + 32 * (2 + 4 * b + 2 * h);
+                const double s2 = (flip && (k & 1)) ? -2.0 * sc : 2.0 * sc;    // eps_k = 2, (-1)^k
+                if (k <= g.K) {
+                    atomicAdd(&o[k].x, (double)v[0] * s2);
+                    atomicAdd(&o[k].y, (double)v[32] * s2);
+                }
+                v[0] = v[32] = 0;
+            }
+        }
+        e = kFaEmpty;
+    };
+
+    unsigned s_next = A.perm[min(wfirst + lane, wlast - 1)];
+    StencilRec64 r_next = A.rec[s_next];
+    double ps_next = A.psi[s_next], y_next = A.y[s_next];
+    for (int64_t t0 = wfirst; t0 < wlast; t0 += 32) {
+        const int cnt = (int)min((int64_t)32, wlast - t0);
+        // ---- 1: one sample per lane
+        const unsigned s = s_next, mycell = r_next.cell;
+        const unsigned prev = __shfl_up_sync(0xffffffffu, mycell, 1);
+        const unsigned heads = __ballot_sync(0xffffffffu, lane < cnt && (lane == 0 || mycell != prev));
+        int ey;                                     // exponent field of the largest |y| of this sample's run
+        long long zc, zs;
+        {
+            double wt[4], wp[4];
+            const int i = (int)(mycell >> 16) - 1, j = (int)(mycell & 0xffffu);
+            fx_weights<4>(g, i, r_next.dth, r_next.fph, wt, wp);
+            long long lwt[4], lwp[4];
+            const double y = y_next;
+            const int yf = (__double2hiint(y) >> 20) & 0x7ff;
+            bool ok = fx_sincos(ps_next, ptab, zc, zs);
+            if (!ok) {                              // |psi| >= 2^9 or not finite
+                double sp, cp;
+                sincos(ps_next, &sp, &cp);
+                ok = fx_q62(cp, zc) && fx_q62(sp, zs);
+            }
+            unsigned long long wsum = 0;            // sum of |wt| in Q60
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                lwt[a] = lwp[a] = 0;
+                ok = fx_q62(wt[a], lwt[a]) && ok;
+                ok = fx_q62(wp[a], lwp[a]) && ok;
+                wsum += (unsigned long long)llabs(lwt[a]) >> 2;
+            }
+            // sum |wt| < 1.5 (1.25 on uniform rings): |wt| < 1.25, so that 512 samples' sums stay
+            // below 2^63
+            ok = ok && wsum < (3ull << 59) && (y == 0.0 || (yf >= 64 && yf <= 1983));
+            if (!ok && lane < cnt) adj_one(A, s);
+            const bool use = ok && lane < cnt && y != 0.0;
+            // the run's largest exponent: runs are contiguous, an inclusive maximum up to its last lane
+            ey = use ? yf : 0;
+            const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, ey, o);
+                if (lane - o >= start) ey = max(ey, v);
+            }
+            const unsigned later = lane < 31 ? heads & (0xfffffffeu << lane) : 0u;
+            ey = __shfl_sync(0xffffffffu, ey, (later ? __ffs(later) - 1 : cnt) - 1);
+            // y w 2^(61 - e), e = ey - 1022; |w| < 2.  Sums over thousands of samples would show a
+            // bias: the first product's truncation (4 units) is centred, the second's is centred by
+            // the digits' rounding, and the sums below round ties to even.
+            const long long yq = use ? fx_from_double(y, ey) >> 1 : 0;
+            __half *arow = reinterpret_cast<__half *>(&W.a[0][0][lane >> 1]) + (lane & 1);
+#pragma unroll 1
+            for (int a = 0; a < 4; ++a) {
+                const long long ya = fx_mul(yq, lwt[0]) + 2;
+                lwt[0] = lwt[1];
+                lwt[1] = lwt[2];
+                lwt[2] = lwt[3];
+#pragma unroll
+                for (int b = 0; b < 4; b += 2) {
+                    uint32_t d[kFxDig];
+                    fx_digits(fx_mul(ya, lwp[b]), fx_mul(ya, lwp[b + 1]), d);
+                    __half *o0 = arow + (4 * a + ((j - 1 + b) & 3)) * (2 * kFaRow);
+                    __half *o1 = arow + (4 * a + ((j + b) & 3)) * (2 * kFaRow);
+#pragma unroll
+                    for (int u = 0; u < kFxDig; ++u) {
+                        const __half2 h = *reinterpret_cast<const __half2 *>(&d[u]);
+                        o0[u * (16 * 2 * kFaRow)] = __low2half(h);
+                        o1[u * (16 * 2 * kFaRow)] = __high2half(h);
+                    }
+                }
+            }
+        }
+        if (t0 + 32 < wlast) {
+            s_next = A.perm[min(t0 + 32 + lane, wlast - 1)];
+            r_next = A.rec[s_next];
+            ps_next = A.psi[s_next];
+            y_next = A.y[s_next];
+        }
+        __half *erow = reinterpret_cast<__half *>(&W.e[0][0][lane >> 1]) + (lane & 1);
+        long long xc = zc, xs = -zs, pc = kFxOne, px = 0;
+        // ---- 2: order 0 (E = 1: the first digit 256 alone, FP16 0x5c00, in column 0), then blocks of
+        // four orders
+        unsigned cell = cur;
+        int e = ecur;
+#pragma unroll 1
+        for (int b = -1; b < nblk; ++b) {
+            if (b >= 0) {
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    uint32_t d[kFxDig];
+                    fx_digits(xc, xs, d);
+#pragma unroll
+                    for (int u = 0; u < kFxDig; ++u) {
+                        const __half2 h = *reinterpret_cast<const __half2 *>(&d[u]);
+                        erow[(u * 8 + 2 * k) * (2 * kFaRow)] = __low2half(h);
+                        erow[(u * 8 + 2 * k + 1) * (2 * kFaRow)] = __high2half(h);
+                    }
+                    const long long nc = (fx_mulhi(zc, xc) << 3) - pc, ns = (fx_mulhi(zc, xs) << 3) - px;
+                    pc = xc;
+                    px = xs;
+                    xc = nc;
+                    xs = ns;
+                }
+            }
+            __syncwarp();
+            cell = cur;
+            e = ecur;
+            long long *v = sums + (b < 0 ? 0 : 32 * (2 + 4 * b));
+            const int nv = b < 0 ? 2 : 4;
+            // runs of equal cells, [r0, r1)
+#pragma unroll 1
+            for (int r0 = 0, r1; r0 < cnt; r0 = r1) {
+                const unsigned rcell = __shfl_sync(0xffffffffu, mycell, r0);
+                const int re = __shfl_sync(0xffffffffu, ey, r0);
+                const unsigned later = r0 < 31 ? heads & (0xfffffffeu << r0) : 0u;
+                r1 = later ? __ffs(later) - 1 : cnt;
+                if (re == 0) continue;              // nothing to add
+                if (rcell != cell) {
+                    if (cell != 0xffffffffu) {
+                        const int jo = (int)(cell & 0xffffu), jn = (int)(rcell & 0xffffu);
+                        const bool near = (rcell >> 16) == (cell >> 16) && jn > jo && jn < jo + 4;
+                        flush(b, cell, e, jo - 1, near ? jn - 1 : jo + 3);
+                    }
+                    cell = rcell;
+                }
+                // sums and contributions to one exponent; the products' unit is 2^(re - 1022 + 1)
+                const int en = re - 1021;
+                int shift = 3;
+                if (en > e) {
+                    if (e != kFaEmpty) {
+                        const int d = min(en - e, 63);
+                        for (int q = 0; q < nv; ++q) v[32 * q] = (v[32 * q] + ((1ll << d) >> 1)) >> d;
+                    }
+                    e = en;
+                } else {
+                    shift = min(3 + e - en, 62);
+                }
+                const long long half = (1ll << (shift - 1)) - 1;
+                float acc[4][kFxSums];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int u = 0; u < kFxSums; ++u) acc[q][u] = 0.f;
+                // the run's samples within each half of the batch
+#pragma unroll 1
+                for (int t = r0 >> 4; t <= (r1 - 1) >> 4; ++t) {
+                    const int p0 = 16 * t + 2 * q4, p1 = p0 + 8;
+                    const uint32_t m0 = (p0 >= r0 && p0 < r1 ? 0xffffu : 0u) | (p0 + 1 >= r0 && p0 + 1 < r1 ? 0xffff0000u : 0u);
+                    const uint32_t m1 = (p1 >= r0 && p1 < r1 ? 0xffffu : 0u) | (p1 + 1 >= r0 && p1 + 1 < r1 ? 0xffff0000u : 0u);
+                    uint32_t ad[kFxDig][4];
+#pragma unroll
+                    for (int u = 0; u < kFxDig; ++u) {
+                        ad[u][0] = W.a[u][gr][8 * t + q4] & m0;
+                        ad[u][1] = W.a[u][gr + 8][8 * t + q4] & m0;
+                        ad[u][2] = W.a[u][gr][8 * t + q4 + 4] & m1;
+                        ad[u][3] = W.a[u][gr + 8][8 * t + q4 + 4] & m1;
+                    }
+                    if (b < 0) {
+                        const uint32_t one = gr == 0 ? 0x5c005c00u : 0u;
+#pragma unroll
+                        for (int u = 0; u < kFxDig; ++u)
+                            mma_f16(acc[0][u], acc[1][u], acc[2][u], acc[3][u], ad[u], one, one);
+                    } else {
+#pragma unroll
+                        for (int w = 0; w < kFxDig; ++w) {
+                            const uint32_t b0 = W.e[w][gr][8 * t + q4], b1 = W.e[w][gr][8 * t + q4 + 4];
+#pragma unroll
+                            for (int u = 0; u < kFxDig; ++u)
+                                if (u < 3 || w < 3)
+                                    mma_f16(acc[0][u + w], acc[1][u + w], acc[2][u + w], acc[3][u + w], ad[u], b0, b1);
+                        }
+                    }
+                }
+                // (row gr, re), (row gr, im), (row gr + 8, re), (row gr + 8, im); order 0: re only
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const long long x = fx_combine(acc[q]), c = (x + half + ((x >> shift) & 1)) >> shift;
+                    if (b >= 0) v[32 * q] += c;
+                    else if (!(q & 1)) v[16 * q] += c;
+                }
+            }
+            __syncwarp();
+        }
+        cur = cell;
+        ecur = e;
+    }
+    if (cur != 0xffffffffu)
+        for (int b = -1; b < nblk; ++b) {
+            int e = ecur;
+            flush(b, cur, e, (int)(cur & 0xffffu) - 1, (int)(cur & 0xffffu) + 3);
+        }
+}
+
+SL_CHECK_READER(chk_interp_adj_fx)
+
+// Two orders share a row of B and a block of four costs 27 mma a run of cells, whatever the run's
+// length, so k_interp_adjoint(_df) stays better where the samples leave few per occupied cell.
+// Equal times, uniform samples: FP64 at 3.4 per cell (K = 16, 1024 x 2048 cells), 10 (K = 8,
+// 256 x 512), 12 (K = 32, 300 x 600); DF64 at 8 (K = 16), 30 (K = 8), 22 (K = 32), 15 (K = 4,
+// 512 x 1024).  The sort's count of occupied cells tells on the device which kernel runs; the
+// other returns at once.  The tiled kernels leave most of the chip idle on small grids and
+// small calls, where this one is always taken: at 127 x 128 cells 153 against 274 us (n = 1e5, K = 4)
+// and 79 against 115 us (3e4, K = 8); at 1024 x 2048, K = 16, 65 against 308 us (n = 1e4).
+// The p = 2 and 6 stencils (4 and 36 nodes) do not fill rows of 16, and above 32 orders the
+// sums no longer leave two blocks a multiprocessor.
+AdjRoute interp_adj_route(const sl_plan *p, int64_t n, float *min_mean) {
+    const bool df = p->precision == SL_DF64;
+    const int64_t cells = (int64_t)(p->R + 1) * p->nphi;
+    *min_mean = (p->K > 8 && p->K <= 16 ? 4.f : 12.f) * (df ? 2.f : 1.f);
+    if (p->p != 4 || p->K > 32) return AdjRoute::tiled;
+    if (n <= (df ? 8192 : 16384) || cells <= 40000 || (double)n >= *min_mean * (double)cells) return AdjRoute::fx;
+    return AdjRoute::by_occupancy;
+}
+
+sl_status launch_interp_adj_fx(sl_plan *p, const SortBufs &b, const double *psi, const double *tod, int64_t n, const unsigned *occ,
+                               float min_mean, double2 *fbar) {
+    FaArgs a;
+    a.g = p->geom;
+    a.psi = psi;
+    a.y = tod;
+    a.rec = (const StencilRec64 *)b.rec;
+    a.perm = b.perm;
+    a.occ = occ;
+    a.min_mean = min_mean;
+    a.n = n;
+    a.fbar = fbar;
+    const size_t sm = 256 * sizeof(longlong2) + kFaWarps * fa_warp_bytes((p->K + 3) / 4);
+    cudaError_t e = allow_dyn_smem(k_interp_adj_fx, sm);
+    if (e != cudaSuccess) return cuda_check(e, "k_interp_adj_fx smem attribute");
+    int nsm = 152, per_sm = 1;
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p->device);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_adj_fx, 32 * kFaWarps, sm);
+    const int64_t full = (int64_t)nsm * std::max(per_sm, 1) * kFaWarps;     // warps of one wave
+    const int64_t waves = std::max<int64_t>(1, (n + full * kFaChunk - 1) / (full * kFaChunk));
+    const int64_t per = (n + full * waves - 1) / (full * waves);            // whole waves
+    a.chunk = (int)(per <= 32 ? std::max<int64_t>(per, 1) : (per + 31) / 32 * 32);
+    const int64_t nwarps = (n + a.chunk - 1) / a.chunk;
+    const int slot = timing_begin(p, "interp_adj_fx");
+    k_interp_adj_fx<<<(unsigned)((nwarps + kFaWarps - 1) / kFaWarps), 32 * kFaWarps, sm, p->stream>>>(a);
+    timing_end(p, slot);
+    return cuda_check(cudaGetLastError(), "k_interp_adj_fx launch");
+}
+
+}  // namespace sl

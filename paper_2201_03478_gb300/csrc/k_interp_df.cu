@@ -26,6 +26,9 @@ struct DfArgs {
     int ntiles, ncell;
     double *tod;       // forward: written; adjoint: the input TOD
     double2 *fbar;     // adjoint cube (adjoint only)
+    const unsigned *occ;   // adjoint, with min_mean: k_interp_adj_fx runs instead if n >= min_mean *occ
+    float min_mean;
+    int64_t n;
 };
 
 __device__ __forceinline__ dfl df_ld(const float2 *p) {
@@ -177,6 +180,7 @@ template <int P>
 __global__ void k_interp_adjoint_df(const DfArgs A) {
     constexpr int NQ = P * P;
     const InterpGeom &g = A.g;
+    if (A.occ && (float)A.n >= A.min_mean * (float)*A.occ) return;
     const int K1 = g.K + 1;
     const int TC = g.tile_cols;
     const int tw = TC + P - 1, th_rows = kTileRows + P - 1, nnode = th_rows * tw;
@@ -321,7 +325,7 @@ size_t interp_adjoint_df_smem_tc(const sl_plan *p, int tc) {
 }
 
 sl_status launch_interp_adjoint_df(sl_plan *p, const SortBufs &b, int fine, const double *psi, const double *tod,
-                                   double2 *fbar) {
+                                   int64_t n, const unsigned *occ, float min_mean, double2 *fbar) {
     if (!b.chunk_off) return set_error(SL_ERR_ARG, "adjoint interpolation needs the per-tile work list");
     DfArgs a;
     a.g = p->geom;
@@ -335,6 +339,9 @@ sl_status launch_interp_adjoint_df(sl_plan *p, const SortBufs &b, int fine, cons
     a.ncell = fine ? kTileRows * p->geom.tile_cols : 1;
     a.tod = const_cast<double *>(tod);   // read only here
     a.fbar = fbar;
+    a.occ = occ;
+    a.min_mean = min_mean;
+    a.n = n;
     const int K1 = p->K + 1;
     const size_t sm = interp_adjoint_df_smem_tc(p, p->geom.tile_cols);
     int nwarps = (K1 + 1) / 2;

@@ -42,6 +42,7 @@
 #include <algorithm>
 
 #include "fxdigits.cuh"
+#include "fxweights.cuh"
 #include "interp_f64.cuh"
 #include "mbar.cuh"
 #include "sl_internal.cuh"
@@ -61,34 +62,6 @@ struct FxRows {
     static constexpr int kWarp = kN * kFxStride * (int)sizeof(long long) + 10 * 32 * (int)sizeof(double2);
     static constexpr size_t bytes = 256 * sizeof(longlong2) + (size_t)kFxWarps * kWarp;
 };
-
-// phi weights of the fraction f in [0, 1): at p = 4 with a = f (f - 1) and b = a - 2 =
-// (f + 1)(f - 2), 8 FP64 operations instead of 15
-template <int P>
-__device__ __forceinline__ void fx_phi_weights(double f, double wp[P]) {
-    if constexpr (P == 4) {
-        const double a = fma(f, f, -f), a6 = a * (1.0 / 6.0), b2 = fma(0.5, a, -1.0);
-        wp[0] = fma(-a6, f, a6 + a6);
-        wp[1] = fma(b2, f, -b2);
-        wp[2] = -b2 * f;
-        wp[3] = fma(a6, f, a6);
-    } else {
-        lagrange_phi<P>(f, wp);
-    }
-}
-
-// x of [-2, 2] in Q62; false when |x| >= 2 or x is NaN
-__device__ __forceinline__ bool fx_q62(double x, long long &v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int ex = (int)(b >> 52) & 0x7ff;
-    if (ex >= 1024) return false;
-    const int sh = 1023 - ex;                        // value = m 2^(ex - 1075), times 2^62
-    const unsigned long long m0 = (b & ((1ull << 52) - 1)) | (1ull << 52);
-    const unsigned long long m = (m0 << 10) >> min(sh, 63);
-    const long long sg = (long long)b >> 63;
-    v = ((long long)m ^ sg) - sg;
-    return true;
-}
 
 // element offset of stencil node q of cell (i, j): ghost rows read their ring at phi + pi
 template <int P>
@@ -119,15 +92,8 @@ __device__ __forceinline__ bool fx_setup(const InterpGeom &g, const StencilRec64
     using Rows = FxRows<P, MB>;
     bool direct = false;
     long long zc, zs;
-    double wt[P], wp[P], o[P], wd[P];
-    const int i = (int)(r.cell >> 16) - 1;
-#pragma unroll
-    for (int a = 0; a < P; ++a) {
-        o[a] = __ldg(g.offs64 + (size_t)(i + 1) * P + a);
-        wd[a] = __ldg(g.wden + (size_t)(i + 1) * P + a);
-    }
-    lagrange_theta<P>(r.dth, o, wd, wt);
-    fx_phi_weights<P>(r.fph, wp);
+    double wt[P], wp[P];
+    fx_weights<P>(g, (int)(r.cell >> 16) - 1, r.dth, r.fph, wt, wp);
     if (!fx_sincos(ps, ptab, zc, zs)) {             // |psi| >= 2^9 or not finite
         double sp, cp;
         sincos(ps, &sp, &cp);

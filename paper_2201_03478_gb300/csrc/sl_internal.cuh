@@ -93,6 +93,7 @@ unsigned chk_sort();
 unsigned chk_interp();
 unsigned chk_interp_df();
 unsigned chk_interp_fx();
+unsigned chk_interp_adj_fx();
 unsigned chk_psigrid();
 unsigned chk_orbital();
 unsigned chk_fft();
@@ -470,11 +471,17 @@ sl_status launch_interp_df(sl_plan *p, const SortBufs &b, int fine, const void *
                            double *tod);
 size_t interp_df_tiled_smem_tc(const sl_plan *p, int tc);
 sl_status launch_interp_adjoint_df(sl_plan *p, const SortBufs &b, int fine, const double *psi, const double *tod,
-                                   double2 *fbar);
+                                   int64_t n, const unsigned *occ, float min_mean, double2 *fbar);
 size_t interp_adjoint_df_smem_tc(const sl_plan *p, int tc);
 // Adjoint scatter over a sort made with rec64 = 1, with_chunks = 1.
 sl_status launch_interp_adjoint(sl_plan *p, const SortBufs &b, int fine, const double *psi, const double *tod,
                                 int64_t n, double2 *fbar);
+// Over a sort by cell: the fixed-point form (k_interp_adj_fx.cu), the tiled one, or both launched
+// and the sort's occupied cells deciding: the fixed-point one if n >= min_mean *occ.
+enum class AdjRoute { tiled, fx, by_occupancy };
+AdjRoute interp_adj_route(const sl_plan *p, int64_t n, float *min_mean);
+sl_status launch_interp_adj_fx(sl_plan *p, const SortBufs &b, const double *psi, const double *tod, int64_t n, const unsigned *occ,
+                               float min_mean, double2 *fbar);
 sl_status launch_ringdft_adjoint(sl_plan *p, const double2 *fbar);
 sl_status launch_lcontract_adjoint(sl_plan *p);
 sl_status launch_lcontract_adj_fx(sl_plan *p);   // over a zeroed Abar (k_adjoint_fx.cu)
