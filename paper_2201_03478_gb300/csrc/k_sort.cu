@@ -10,7 +10,7 @@
 //
 //   k_bin:        pointing -> (i, j) in double; key; record {theta - theta(i-1),
 //                 phi fraction, [reduced psi], cell}; key histogram
-//   k_scan_local / k_scan1 / k_scan_add:  exclusive prefix sum of the histogram
+//   k_scan_local / k_scan_add:  exclusive prefix sum of the histogram
 //                 -> first position of every key (and a cursor copy)
 //   k_scatter_agg: perm[cursor[key]++] = s, the cursor atomics aggregated per
 //                 chunk of samples in shared memory (order within a key unspecified)
@@ -143,60 +143,79 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned &e
     return tot;
 }
 
-// Per CTA: exclusive scan of data[b*4096 .. +4096) in place, block total to bsum[b], the
-// number of nonzero entries to nz[b].
+// Sum of x over the CTA (1024 threads), in every thread.
+__device__ __forceinline__ unsigned block_sum(unsigned x) {
+    __shared__ unsigned s_part[32];
+    x = __reduce_add_sync(0xffffffffu, x);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = x;
+    __syncthreads();
+    x = __reduce_add_sync(0xffffffffu, s_part[threadIdx.x & 31]);
+    __syncthreads();
+    return x;
+}
+
+// Four words from data + base on (zero from n on), one 16-byte access where data is aligned.
+__device__ __forceinline__ uint4 load4(const unsigned *data, int64_t base, int64_t n) {
+    if (base + 3 < n && ((uintptr_t)data & 15) == 0) return *reinterpret_cast<const uint4 *>(data + base);
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (base < n) v.x = data[base];
+    if (base + 1 < n) v.y = data[base + 1];
+    if (base + 2 < n) v.z = data[base + 2];
+    if (base + 3 < n) v.w = data[base + 3];
+    return v;
+}
+__device__ __forceinline__ void store4(unsigned *data, int64_t base, int64_t n, uint4 v) {
+    if (base + 3 < n && ((uintptr_t)data & 15) == 0) {
+        *reinterpret_cast<uint4 *>(data + base) = v;
+        return;
+    }
+    if (base < n) data[base] = v.x;
+    if (base + 1 < n) data[base + 1] = v.y;
+    if (base + 2 < n) data[base + 2] = v.z;
+    if (base + 3 < n) data[base + 3] = v.w;
+}
+
+// Per CTA: exclusive scan of data[b*4096 .. +4096) in place, block total to bsum[b] and, with nz,
+// the number of nonzero entries to nz[b].
 __global__ void __launch_bounds__(1024) k_scan_local(int64_t n, unsigned *__restrict__ data,
                                                       unsigned *__restrict__ bsum, unsigned *__restrict__ nz) {
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + 4 * threadIdx.x;
-    unsigned v[4], t = 0;
-    int nonzero = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        v[q] = (base + q < n) ? data[base + q] : 0u;
-        t += v[q];
-        nonzero += __syncthreads_count(v[q] != 0u);
-    }
+    const uint4 v = load4(data, base, n);
     unsigned ex;
-    const unsigned tot = block_exclusive_scan(t, ex);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if (base + q < n) data[base + q] = ex;
-        ex += v[q];
-    }
+    const unsigned tot = block_exclusive_scan(v.x + v.y + v.z + v.w, ex);
+    store4(data, base, n, make_uint4(ex, ex + v.x, ex + v.x + v.y, ex + v.x + v.y + v.z));
+    const unsigned nonzero = nz ? block_sum((v.x != 0u) + (v.y != 0u) + (v.z != 0u) + (v.w != 0u)) : 0u;
     if (threadIdx.x == 0) {
         bsum[blockIdx.x] = tot;
-        nz[blockIdx.x] = (unsigned)nonzero;
+        if (nz) nz[blockIdx.x] = nonzero;
     }
 }
 
-// Single CTA: exclusive scan of data[0..n) in place; data[n] = total.  With occ, also
-// *occ = the sum of nz[0..n).
-__global__ void __launch_bounds__(1024) k_scan1(int n, unsigned *__restrict__ data, const unsigned *__restrict__ nz,
-                                                unsigned *__restrict__ occ) {
-    unsigned carry = 0, occupied = 0;
-    for (int base = 0; base < n; base += 1024) {
-        const int t = base + threadIdx.x;
-        const unsigned v = (t < n) ? data[t] : 0u;
-        unsigned ex;
-        const unsigned tot = block_exclusive_scan(v, ex);
-        if (t < n) data[t] = carry + ex;
-        carry += tot;
-        if (occ) occupied += block_exclusive_scan((t < n) ? nz[t] : 0u, ex);
+// Adds the totals of the CTAs before to k_scan_local's sums and copies them to cursor; the
+// last CTA also writes data[n] = total and, with occ, *occ = the sum of nz.  Every CTA sums the
+// earlier totals itself (nb^2 / 2 words from L2, 0.5 MB at 1024 x 2048 cells): a scan of them by
+// one CTA in between, and of the tiles' chunks by another, cost the small and sparse sorts two
+// launches, and with the tiles' strided words more than the rest of the scan (1500 x 3000
+// cells: 17 + 5 + 12 + 4 + 66 us; both kernels now 17 us at 1024 x 2048, 24 before).
+__global__ void __launch_bounds__(1024) k_scan_add(int64_t n, unsigned *__restrict__ data, const unsigned *__restrict__ bsum,
+                                                    const unsigned *__restrict__ nz, unsigned *__restrict__ cursor,
+                                                    unsigned *__restrict__ occ) {
+    const int64_t base = (int64_t)blockIdx.x * kScanBlock + 4 * threadIdx.x;
+    uint4 v = load4(data, base, n);
+    unsigned before = 0;
+    for (unsigned i = threadIdx.x; i < blockIdx.x; i += 1024) before += bsum[i];
+    before = block_sum(before);
+    v = make_uint4(before + v.x, before + v.y, before + v.z, before + v.w);
+    store4(data, base, n, v);
+    store4(cursor, base, n, v);
+    if (blockIdx.x != gridDim.x - 1) return;
+    if (occ) {
+        unsigned o = 0;
+        for (unsigned i = threadIdx.x; i < gridDim.x; i += 1024) o += nz[i];
+        o = block_sum(o);
+        if (threadIdx.x == 0) *occ = o;
     }
-    if (threadIdx.x == 0) {
-        data[n] = carry;
-        if (occ) *occ = occupied;
-    }
-}
-
-__global__ void k_scan_add(int64_t n, unsigned *__restrict__ data, const unsigned *__restrict__ bsum,
-                           unsigned *__restrict__ cursor, unsigned total_slot_from_bsum) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned v = data[i] + bsum[i / kScanBlock];
-        data[i] = v;
-        cursor[i] = v;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) data[n] = bsum[total_slot_from_bsum];
+    if (threadIdx.x == 0) data[n] = before + bsum[blockIdx.x];
 }
 
 // The scatter with its atomics aggregated per chunk of kAggChunk samples: a
@@ -208,64 +227,72 @@ __global__ void k_scan_add(int64_t n, unsigned *__restrict__ data, const unsigne
 // chunk holds about two visits of every cell of a circle; a per-lane scatter
 // (one returning atomic per run of equal keys in a warp) waited for one
 // round trip per warp and 32 samples.
-constexpr int kAggThreads = 256, kAggPer = 16, kAggChunk = kAggThreads * kAggPer;
-constexpr int kAggLog = 13, kAggSlots = 1 << kAggLog;   // > 2 x the distinct keys of a chunk
-static_assert(kAggSlots >= kAggChunk, "the hash table must hold every distinct key of a chunk");
+// PER samples a thread: 16 where that fills the chip; 2 below, so that a short TOD spreads over
+// more CTAs and each clears and walks an eighth of the table (1e5 uniform samples 22 -> 8 us, 1e6 29
+// -> 20; from 1.2e6 on the larger chunk's fewer global atomics are as good: 3e6 65 us).
+constexpr int kAggThreads = 256;
+constexpr int agg_chunk(int per) { return kAggThreads * per; }
+constexpr int agg_log(int per) { return per == 16 ? 13 : 10; }   // slots: 2 x the chunk's samples
+static_assert((1 << agg_log(16)) == 2 * agg_chunk(16) && (1 << agg_log(2)) == 2 * agg_chunk(2),
+              "the hash table must hold every distinct key of a chunk");
 constexpr unsigned kNoKey = 0xffffffffu;
 
+template <int PER>
 __global__ void __launch_bounds__(kAggThreads) k_scatter_agg(int64_t n, int64_t nkeys, const unsigned *__restrict__ keys,
                                                              unsigned *__restrict__ cursor,
                                                              unsigned *__restrict__ perm) {
+    constexpr int CHUNK = agg_chunk(PER), LOG = agg_log(PER), SLOTS = 1 << LOG;
+    constexpr int NQ = SLOTS / kAggThreads < 8 ? SLOTS / kAggThreads : 8;   // atomics in flight a thread
     extern __shared__ __align__(16) unsigned agg_smem[];
-    unsigned *hkey = agg_smem, *hval = agg_smem + kAggSlots;   // key per slot; count, then range start
-    const int64_t per = (n + (int64_t)gridDim.x * kAggChunk - 1) / ((int64_t)gridDim.x * kAggChunk) * kAggChunk;
+    unsigned *hkey = agg_smem, *hval = agg_smem + SLOTS;   // key per slot; count, then range start
+    const int64_t per = (n + (int64_t)gridDim.x * CHUNK - 1) / ((int64_t)gridDim.x * CHUNK) * CHUNK;
     const int64_t sbeg = min(n, (int64_t)blockIdx.x * per), send = min(n, sbeg + per);
-    for (int64_t c0 = sbeg; c0 < send; c0 += kAggChunk) {
-        for (int i = threadIdx.x; i < kAggSlots / 4; i += kAggThreads) {
+    for (int64_t c0 = sbeg; c0 < send; c0 += CHUNK) {
+        for (int i = threadIdx.x; i < SLOTS / 4; i += kAggThreads) {
             reinterpret_cast<uint4 *>(hkey)[i] = make_uint4(kNoKey, kNoKey, kNoKey, kNoKey);
             reinterpret_cast<uint4 *>(hval)[i] = make_uint4(0u, 0u, 0u, 0u);
         }
         __syncthreads();
-        unsigned slot[kAggPer], rank[kAggPer];
+        unsigned slot[PER], rank[PER];
 #pragma unroll
-        for (int j = 0; j < kAggPer; ++j) {
+        for (int j = 0; j < PER; ++j) {
             const int64_t s = c0 + (int64_t)j * kAggThreads + threadIdx.x;
-            slot[j] = kAggSlots;
+            slot[j] = SLOTS;
             rank[j] = 0u;
             if (s < send) {
                 unsigned key = keys[s];
                 if (!SL_GUARD(key < nkeys, 0x102u)) key = 0;
-                unsigned h = (key * 2654435761u) >> (32 - kAggLog);
+                unsigned h = (key * 2654435761u) >> (32 - LOG);
                 // linear probing; the table holds more slots than the chunk has samples,
-                // so a free or matching slot is always found within kAggSlots probes
-                for (int probe = 0; probe < kAggSlots; ++probe) {
+                // so a free or matching slot is always found within SLOTS probes
+                for (int probe = 0; probe < SLOTS; ++probe) {
                     const unsigned prev = atomicCAS(&hkey[h], kNoKey, key);
                     if (prev == kNoKey || prev == key) break;
-                    h = (h + 1u) & (kAggSlots - 1);
+                    h = (h + 1u) & (SLOTS - 1);
                 }
                 slot[j] = h;
                 rank[j] = atomicAdd(&hval[h], 1u);
             }
         }
         __syncthreads();
-        for (int i0 = threadIdx.x; i0 < kAggSlots; i0 += 8 * kAggThreads) {
-            unsigned got[8];
+        for (int i0 = threadIdx.x; i0 < SLOTS; i0 += NQ * kAggThreads) {
+            unsigned got[NQ];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const int i = i0 + q * kAggThreads;
                 const unsigned k = hkey[i];
                 got[q] = (k != kNoKey) ? atomicAdd(cursor + k, hval[i]) : 0u;
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < NQ; ++q) {
                 const int i = i0 + q * kAggThreads;
                 if (hkey[i] != kNoKey) hval[i] = got[q];
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int j = 0; j < kAggPer; ++j) {
-            if (slot[j] >= kAggSlots) continue;
+        for (int j = 0; j < PER; ++j) {
+            if (slot[j] >= SLOTS) continue;
             const int64_t s = c0 + (int64_t)j * kAggThreads + threadIdx.x;
             const unsigned pos = hval[slot[j]] + rank[j];
             if (SL_GUARD(pos < n, 0x103u)) perm[pos] = (unsigned)s;
@@ -274,16 +301,28 @@ __global__ void __launch_bounds__(kAggThreads) k_scatter_agg(int64_t n, int64_t 
     }
 }
 
-// chunk_off[t] = ceil(#samples of tile t / kChunk); scanned by k_scan1 afterwards.
-__global__ void k_tile_chunks(int ntiles, int ncell, const unsigned *__restrict__ start,
-                              unsigned *__restrict__ chunk_off) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntiles) return;
-    const unsigned c = start[(int64_t)(t + 1) * ncell] - start[(int64_t)t * ncell];
-    chunk_off[t] = (c + kChunk - 1) / kChunk;
+// chunk_off[t] = sum over the tiles before t of ceil(#samples / kChunk), chunk_off[ntiles] = total.
+// One CTA per 1024 tiles, which also sums the chunks of the tiles before its own (up to 64
+// strided rounds of independent loads at the largest grids).
+__global__ void __launch_bounds__(1024) k_tile_chunks(int ntiles, int ncell, const unsigned *__restrict__ start,
+                                                       unsigned *__restrict__ chunk_off) {
+    auto chunks = [&](int t) {
+        return (start[(int64_t)(t + 1) * ncell] - start[(int64_t)t * ncell] + kChunk - 1) / kChunk;
+    };
+    const int t0 = blockIdx.x * 1024, t = t0 + threadIdx.x;
+    unsigned before = 0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < t0; i += 1024) before += chunks(i);
+    before = block_sum(before);
+    unsigned ex;
+    const unsigned tot = block_exclusive_scan(t < ntiles ? chunks(t) : 0u, ex);
+    if (t < ntiles) chunk_off[t] = before + ex;
+    if (threadIdx.x == 0 && t0 + 1024 >= ntiles) chunk_off[ntiles] = before + tot;
 }
 
 SL_CHECK_READER(chk_sort)
+
+constexpr int kAggFull = 304;   // chunks of 4096 samples that fill the chip (two CTAs an SM)
 
 static unsigned grid_for(int64_t n, int bs) {
     int64_t b = (n + bs - 1) / bs;
@@ -311,25 +350,26 @@ sl_status launch_sort_into(sl_plan *p, const SortBufs &b, const double *theta, c
     timing_end(p, slot);
     if ((st = cuda_check(cudaGetLastError(), "k_bin launch")) != SL_OK) return st;
     slot = timing_begin(p, "scan");
-    k_scan_local<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, b.cursor);
-    k_scan1<<<1, 1024, 0, p->stream>>>((int)nb, b.bsum, b.cursor, b.occ);
-    k_scan_add<<<(unsigned)std::min<int64_t>((nkeys + 255) / 256, 152 * 16), 256, 0, p->stream>>>(
-        nkeys, b.hist, b.bsum, b.cursor, (unsigned)nb);
+    unsigned *nz = b.occ ? b.occ + 1 : nullptr;
+    k_scan_local<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, nz);
+    k_scan_add<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, nz, b.cursor, b.occ);
     timing_end(p, slot);
     if ((st = cuda_check(cudaGetLastError(), "k_scan launch")) != SL_OK) return st;
     slot = timing_begin(p, "scatter");
     {
-        const size_t sm = 2 * (size_t)kAggSlots * sizeof(unsigned);
-        if ((st = cuda_check(allow_dyn_smem(k_scatter_agg, sm), "k_scatter_agg smem attribute")) != SL_OK) return st;
-        const int64_t nchunk = (n + kAggChunk - 1) / kAggChunk;
+        const bool big = n >= (int64_t)kAggFull * agg_chunk(16);
+        auto kern = big ? k_scatter_agg<16> : k_scatter_agg<2>;
+        const int chunk = agg_chunk(big ? 16 : 2);
+        const size_t sm = 4 * (size_t)chunk * sizeof(unsigned);
+        if ((st = cuda_check(allow_dyn_smem(kern, sm), "k_scatter_agg smem attribute")) != SL_OK) return st;
+        const int64_t nchunk = (n + chunk - 1) / chunk;
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nchunk, 152 * 3 * 4));
-        k_scatter_agg<<<grid, kAggThreads, sm, p->stream>>>(n, nkeys, b.keys, b.cursor, b.perm);
+        kern<<<grid, kAggThreads, sm, p->stream>>>(n, nkeys, b.keys, b.cursor, b.perm);
     }
     timing_end(p, slot);
     if ((st = cuda_check(cudaGetLastError(), "k_scatter_agg launch")) != SL_OK) return st;
     if (with_chunks) {
-        k_tile_chunks<<<(p->ntiles + 255) / 256, 256, 0, p->stream>>>(p->ntiles, ncell, b.hist, b.chunk_off);
-        k_scan1<<<1, 1024, 0, p->stream>>>(p->ntiles, b.chunk_off, nullptr, nullptr);
+        k_tile_chunks<<<(p->ntiles + 1023) / 1024, 1024, 0, p->stream>>>(p->ntiles, ncell, b.hist, b.chunk_off);
         st = cuda_check(cudaGetLastError(), "k_tile_chunks launch");
     }
     return st;

@@ -154,7 +154,7 @@ static sl_status alloc_sort_tables(sl_plan *p) {
     p->nkeys = sort_nkeys(p, 1);
     sl_status st = dalloc_t(p, &p->sort.hist, (size_t)p->nkeys + 1, "cell histogram");
     if (st == SL_OK) st = dalloc_t(p, &p->sort.cursor, (size_t)p->nkeys, "cell cursor");
-    if (st == SL_OK) st = dalloc_t(p, &p->sort.bsum, (size_t)sort_nbsum(p->nkeys) + 2, "scan block sums");
+    if (st == SL_OK) st = dalloc_t(p, &p->sort.bsum, 2 * (size_t)sort_nbsum(p->nkeys) + 2, "scan block sums");
     if (st == SL_OK) p->sort.occ = p->sort.bsum + sort_nbsum(p->nkeys) + 1;
     if (st == SL_OK) st = dalloc_t(p, &p->sort.chunk_off, (size_t)p->ntiles + 1, "tile chunks");
     return st;
@@ -166,7 +166,7 @@ static void free_sort_tables(sl_plan *p) {
     dfree(p->sort.bsum);
     dfree(p->sort.chunk_off);
     p->sort.hist = p->sort.cursor = p->sort.bsum = p->sort.chunk_off = p->sort.occ = nullptr;
-    p->bytes_held -= (int64_t)sizeof(unsigned) * ((p->nkeys + 1) + p->nkeys + (sort_nbsum(p->nkeys) + 2) +
+    p->bytes_held -= (int64_t)sizeof(unsigned) * ((p->nkeys + 1) + p->nkeys + (2 * sort_nbsum(p->nkeys) + 2) +
                                                   (p->ntiles + 1));
 }
 

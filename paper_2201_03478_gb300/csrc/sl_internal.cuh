@@ -224,9 +224,9 @@ struct SortBufs {
     void *rec;            // [n] StencilRec64 or StencilRec32, by sample
     unsigned *hist;       // [nkeys + 1]: key counts, then first position of each key
     unsigned *cursor;     // [nkeys]
-    unsigned *bsum;       // [nkeys / 4096 + 2]
+    unsigned *bsum;       // [nkeys / 4096 + 2], with occ twice that
     unsigned *chunk_off;  // [ntiles + 1]
-    unsigned *occ;        // keys that hold samples (in bsum's last entry; written by the sort)
+    unsigned *occ;        // keys that hold samples (behind the block sums, their parts following it; written by the sort), or null
 };
 
 // Rescaled l-recurrence coefficients per (k, m, l), stored at
