@@ -346,22 +346,22 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
 
 SL_CHECK_READER(chk_interp_adj_fx)
 
-// Two orders share a row of B and a block of four costs 27 mma a run of cells, whatever the run's
-// length, so k_interp_adjoint(_df) stays better where the samples leave few per occupied cell.
-// Equal times, uniform samples: FP64 at 3.4 per cell (K = 16, 1024 x 2048 cells), 10 (K = 8,
-// 256 x 512), 12 (K = 32, 300 x 600); DF64 at 8 (K = 16), 30 (K = 8), 22 (K = 32), 15 (K = 4,
-// 512 x 1024).  The sort's count of occupied cells tells on the device which kernel runs; the
-// other returns at once.  The tiled kernels leave most of the chip idle on small grids and
-// small calls, where this one is always taken: at 127 x 128 cells 153 against 274 us (n = 1e5, K = 4)
-// and 79 against 115 us (3e4, K = 8); at 1024 x 2048, K = 16, 65 against 308 us (n = 1e4).
-// The p = 2 and 6 stencils (4 and 36 nodes) do not fill rows of 16, and above 32 orders the
-// sums no longer leave two blocks a multiprocessor.
+// A block of four orders costs 27 mma a run of cells, whatever the run's length, so
+// k_interp_adjoint(_df) stays better where the samples leave few per occupied cell.  Equal times,
+// uniform samples: FP64 at 3.4 per cell (K = 16, 1024 x 2048 cells), 10 (K = 8, 256 x 512; K = 16
+// there: 1.43 at 7.6), 12 (K = 32, 300 x 600); DF64 at 8 (K = 16, 1024 x 2048), 30 (K = 8), 22 (K =
+// 32), 15 (K = 4, 512 x 1024).  The sort's count of occupied cells tells on the device which
+// kernel runs; the other returns at once.  The tiled kernels leave most of the chip idle on
+// small grids and small calls, where this one is always taken: at 127 x 128 cells 153 against 274 us
+// (n = 1e5, K = 4) and 79 against 115 us (3e4, K = 8; DF64 loses above 4 orders: 1.25 at K = 6, 3e5);
+// at 1024 x 2048, K = 16, 65 against 308 us (n = 1e4).  The p = 2 and 6 stencils (4 and 36 nodes) do
+// not fill rows of 16, and above 32 orders the sums no longer leave two blocks a multiprocessor.
 AdjRoute interp_adj_route(const sl_plan *p, int64_t n, float *min_mean) {
     const bool df = p->precision == SL_DF64;
     const int64_t cells = (int64_t)(p->R + 1) * p->nphi;
-    *min_mean = (p->K > 8 && p->K <= 16 ? 4.f : 12.f) * (df ? 2.f : 1.f);
+    *min_mean = df ? 24.f : 12.f;
     if (p->p != 4 || p->K > 32) return AdjRoute::tiled;
-    if (n <= (df ? 8192 : 16384) || cells <= 40000 || (double)n >= *min_mean * (double)cells) return AdjRoute::fx;
+    if (n <= (df ? 8192 : 16384) || (cells <= 40000 && p->K <= (df ? 4 : 16)) || (double)n >= *min_mean * (double)cells) return AdjRoute::fx;
     return AdjRoute::by_occupancy;
 }
 

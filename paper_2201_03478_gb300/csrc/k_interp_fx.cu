@@ -430,6 +430,8 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
 // of 32 samples as there, the phases split into halves per lane beforehand; then sample by
 // sample, each lane 2 nodes x 4 orders: F as (xh, xl), kept while the cell stays the same,
 // three multiply-adds per real term, sums over the quad by shuffles, weights as there.
+// NE blocks of four orders: with fewer, more warps fit (4 CTAs an SM up to 8 orders, 3 above:
+// 403 -> 319 us at K = 4, 1e6 samples in as many cells); small calls take fewer samples a warp.
 // The next cell's nodes are loaded while the current sample is summed.  Bound by the
 // integer pipe (20 instructions per real value of F); the cube is read in 64-byte pieces
 // per quad, where one sample per thread reads 16-byte pieces from 32 lines at a time and
@@ -438,11 +440,12 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
 constexpr int kFxsWarps = 4;
 constexpr int kFxsPhStride = 33;   // 16-byte entries per order: a quad's 4 orders in distinct banks
 
-__global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __grid_constant__ InterpGeom g,
+template <int NE>
+__global__ void __launch_bounds__(32 * kFxsWarps, NE <= 2 ? 4 : 3) k_interp_fx_short(const __grid_constant__ InterpGeom g,
                                                                        const double2 *__restrict__ maps,
                                                                        const StencilRec64 *__restrict__ rec,
                                                                        const double *__restrict__ psi,
-                                                                       const unsigned *__restrict__ perm, int64_t n,
+                                                                       const unsigned *__restrict__ perm, int64_t n, int bs,
                                                                        const unsigned *__restrict__ occ, float min_mean,
                                                                        double *__restrict__ tod) {
     if (!((float)n < min_mean * (float)*occ)) return;       // k_interp_fx runs instead
@@ -453,16 +456,16 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
     for (int q = threadIdx.x; q < 256; q += 32 * kFxsWarps) ptab[q] = __ldg(g.phase_tab + q);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int4 *ph = reinterpret_cast<int4 *>(fx_smem + 256 * sizeof(longlong2)) + (size_t)warp * 16 * kFxsPhStride;
+    int4 *ph = reinterpret_cast<int4 *>(fx_smem + 256 * sizeof(longlong2)) + (size_t)warp * 4 * NE * kFxsPhStride;
     long long *tab = reinterpret_cast<long long *>(fx_smem + 256 * sizeof(longlong2) +
-                                                   (size_t)kFxsWarps * 16 * kFxsPhStride * sizeof(int4)) +
+                                                   (size_t)kFxsWarps * 4 * NE * kFxsPhStride * sizeof(int4)) +
                      (size_t)warp * Rows::kN * kFxStride;
     const int gr = lane >> 2, q4 = lane & 3;
     const int K = g.K;
-    const int64_t nbatch = (n + 31) / 32;
+    const int64_t nbatch = (n + bs - 1) / bs;
     for (int64_t batch = (int64_t)blockIdx.x * kFxsWarps + warp; batch < nbatch; batch += (int64_t)gridDim.x * kFxsWarps) {
-        const int64_t t0 = batch * 32;
-        const int cnt = (int)min((int64_t)32, n - t0);
+        const int64_t t0 = batch * bs;
+        const int cnt = (int)min((int64_t)bs, n - t0);
         const unsigned s = perm[t0 + min(lane, cnt - 1)];
         unsigned mycell;
         bool direct;
@@ -476,7 +479,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
         for (int q = 0; q < 4; ++q) {
             FxPhase f(tab + lane, Rows::kC4, q, 0);
 #pragma unroll 1
-            for (int e = 0; e < 4 && 4 * e + q < K; ++e) {
+            for (int e = 0; e < NE && 4 * e + q < K; ++e) {
                 int4 v;
                 fx_split(f.c, v.x, v.y);
                 fx_split(f.s, v.z, v.w);
@@ -487,9 +490,9 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
         __syncwarp();
         unsigned a_cell = 0xffffffffu;
         int a_ef = 0;
-        int ah[2][4][2], al[2][4][2];
+        int ah[2][NE][2], al[2][NE][2];
         long long f0[2] = {0, 0};
-        double2 raw[2][4];
+        double2 raw[2][NE];
         double raw0[2];
         auto fetch = [&](unsigned cell) {
             const int i = (int)(cell >> 16) - 1, j = (int)(cell & 0xffffu);
@@ -498,7 +501,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
                 const double2 *src = maps + fx_node<P>(g, i, j, gr + 8 * h);
                 raw0[h] = __ldg(&src->x);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
+                for (int e = 0; e < NE; ++e) {
                     const int k = q4 + 1 + 4 * e;
                     raw[h][e] = k <= K ? __ldg(src + k) : make_double2(0.0, 0.0);
                 }
@@ -514,7 +517,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
                 for (int h = 0; h < 2; ++h) {
                     mx = max(mx, (uint32_t)__double2hiint(raw0[h]) & 0x7fffffffu);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
+                    for (int e = 0; e < NE; ++e)
                         mx = max(mx, max((uint32_t)__double2hiint(raw[h][e].x) & 0x7fffffffu,
                                          (uint32_t)__double2hiint(raw[h][e].y) & 0x7fffffffu));
                 }
@@ -529,7 +532,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
                         const bool flip = (row < 0 || row >= g.R) && !(q4 & 1);
                         f0[h] = fx_from_double(raw0[h], a_ef) >> 6;
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
+                        for (int e = 0; e < NE; ++e) {
                             if (4 * e >= K) continue;
                             long long x = fx_from_double(raw[h][e].x, a_ef), y = fx_from_double(raw[h][e].y, a_ef);
                             if (flip) { x = -x; y = -y; }
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
             if (a_ef == 2047) continue;
             long long hh[2] = {0, 0}, xx[2] = {0, 0};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
+            for (int e = 0; e < NE; ++e) {
                 if (4 * e >= K) continue;
                 // orders past K: F is zero there, and so is the product with whatever ph holds
                 const int4 y = ph[(4 * e + q4) * kFxsPhStride + c];
@@ -584,30 +587,42 @@ __global__ void __launch_bounds__(32 * kFxsWarps, 3) k_interp_fx_short(const __g
     }
 }
 
-static size_t fx_short_smem() {
-    return 256 * sizeof(longlong2) +
-           (size_t)kFxsWarps * (16 * kFxsPhStride * sizeof(int4) + FxRows<4, false>::kN * kFxStride * sizeof(long long));
+static size_t fx_short_smem(int ne) {
+    return 256 * sizeof(longlong2) + (size_t)kFxsWarps * (4 * ne * kFxsPhStride * sizeof(int4) +
+                                                          FxRows<4, false>::kN * kFxStride * sizeof(long long));
 }
 
 SL_CHECK_READER(chk_interp_fx)
 
-// Which calls take the fixed-point sums.  At p = 4 and K <= 16, FP64 plans always: the two
-// kernels cover few and many samples per cell (K = 16, LFI-size grid, ms, direct FP64 sum in
-// brackets: 1e8 scan samples 18.2 [108.7], 1e7 uniform ones on 2e6 cells 6.2 [10.9], 1e6:
-// 1.09 [1.12]; one 55-minute period: 0.051 [0.133]).  For p = 2 and 6 and beyond 16 orders
-// there is only the tensor-core form, whose operands cost several row tiles or blocks per
-// cell: from 48 samples per grid cell on (K = 32, p = 6, 55 per cell: 22 [43]; 5.5 per cell:
-// 11 [4.4]; K = 8, p = 2: 1.6 [2.3] and 0.60 [0.24]).  DF64 plans have the double-float
-// kernel instead of the direct sum: p = 4, K <= 16 from 8 samples per grid cell on (1e8 scan
-// samples 18.2 [32.0]; 2e7: 3.6 [6.4]; 1e7 uniform ones: 6.2 [4.1]).  Grid cells, not
-// occupied ones, and the whole TOD's samples, so that the choice is known to the host and
-// every piece of a TOD gets the same kernel.
+constexpr int64_t kFxFew = 20480;   // some 8 samples a warp of k_interp_fx
+
+// Which calls take the fixed-point sums (FP64 plans otherwise k_interp_f64, DF64 plans
+// k_interp_df).  A cell's operand costs the same at every K, so few orders need many samples per
+// cell.  At p = 4 the line is the density of uniform samples (the slowest form: a scan fills
+// fewer cells) at which they break even (time over the direct sum's, FP64, 127 x 128, 256 x
+// 512 and 1024 x 2048 cells): K = 1 1.19, 0.86 at 61 and 122 per cell; K = 2 1.19, 0.94 at 37 and
+// 61; K = 3 1.26, 0.89 at 6 and 12; K = 4 1.02, 0.84 at 2.3 and 4.6; K = 8 1.14, 0.89 at 0.5 and
+// 1.4; K = 12 1.10, 0.80 at 0.14 and 1.4; K = 16 1.09, 0.76 (a 55-minute scan period: 0.39).
+// K = 0 gains nothing.  With at most some 8 samples for every warp of the chip, the products of
+// a cell take less time than one thread's sums: from 4 orders on 12 against 21 us (1000 samples; uniform
+// ones even out at 7e3 with K = 4 and at 1.4e4 with K = 8; a scan still gains a fifth at 2e4).
+// For p = 2 and 6 and beyond 16 orders there is only the tensor-core
+// form, whose operands cost several row tiles or blocks per cell: from 48 samples per grid
+// cell on (K = 32, p = 6, 55 per cell: 22 [43] ms; 5.5 per cell: 11 [4.4]; K = 8, p = 2: 1.6 [2.3]
+// and 0.60 [0.24]), 96 below 8 orders (K = 4: 1.26 at 61, 0.91 at 122), none below 3 (K = 2: 1.2 at 122).  DF64's alternative is faster: 13 to 16 orders from 8 samples per cell on
+// (1e8 scan samples 18.2 [32.0]; 2e7: 3.6 [6.4]; uniform ones break even at 60 per cell, 1.18 at
+// 23), 8 orders lose 1.35 at 61 per cell.  Grid cells, not occupied ones, and the whole TOD's
+// samples, so that the choice is known to the host and every piece of a TOD gets the same
+// kernel.
 bool interp_uses_fx(const sl_plan *p, int64_t n_total) {
     if (plan_fp32(p->precision)) return false;
-    const bool base = p->p == 4 && p->K <= 16;
     const double per_cell = (double)n_total / ((double)(p->R + 1) * p->nphi);
-    if (p->precision == SL_DF64) return base && per_cell >= 8.0;
-    return base || per_cell >= 48.0;
+    if (p->precision == SL_DF64) return p->p == 4 && p->K > 12 && p->K <= 16 && per_cell >= 8.0;
+    if (p->p != 4 || p->K > 16) return p->K > 2 && per_cell >= (p->K < 8 ? 96.0 : 48.0);
+    if (p->K == 0) return false;
+    if (p->K >= 4 && n_total <= kFxFew) return true;
+    constexpr double kLine[11] = {0.0, 96.0, 48.0, 8.0, 4.0, 4.0, 4.0, 4.0, 2.0, 2.0, 2.0};
+    return p->K > 10 || per_cell >= kLine[p->K];
 }
 
 sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n, double *tod) {
@@ -634,21 +649,26 @@ sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, cons
     const int64_t waves = std::max<int64_t>(1, (n + full * 512 - 1) / (full * 512));
     const int64_t per = (n + full * waves - 1) / (full * waves);  // whole waves
     const int chunk = (int)(per <= 32 ? std::max<int64_t>(per, 1) : (per + 31) / 32 * 32);
-    // Few samples per occupied cell take less time in k_interp_fx_short (K = 16: equal at 5; at
-    // 0.5, 1.08 and 1.94 ms; K = 4: at 6, 0.059 and 0.106 ms, at 61, 0.32 and 0.27 ms).  When
-    // that may be the case and the call is large enough to fill the SMs both are launched, and
-    // the sort's count of occupied cells decides on the device which one runs (the other
-    // returns at once).
-    const float kMean = p->K <= 8 ? 10.f : 5.f;
+    // Few samples per occupied cell take less time in k_interp_fx_short (equal at 23: K = 16, 3e6
+    // samples on 256 x 512 cells 1.46 and 1.49 ms; at 12, 2e5 on 127 x 128: 0.20 and 0.13 ms; K = 4 at
+    // 15, 2e6: 0.87 and 0.66).  When that may be the case and the call is large enough to fill
+    // the SMs both are launched, and the sort's count of occupied cells decides on the device
+    // which one runs (the other returns at once).
+    constexpr float kMean = 24.f;
     const bool both = p->p == 4 && !mb && n > 4 * full && (float)n < kMean * (float)p->nkeys;
     if (both) {
-        const size_t sm_short = fx_short_smem();
-        e = allow_dyn_smem(k_interp_fx_short, sm_short);
+        const int ne = std::max(1, (p->K + 3) / 4), ctas = nsm * (ne <= 2 ? 4 : 3);
+        auto short_kern = ne == 1 ? k_interp_fx_short<1> : ne == 2 ? k_interp_fx_short<2> : ne == 3 ? k_interp_fx_short<3>
+                                                                                         : k_interp_fx_short<4>;
+        const size_t sm_short = fx_short_smem(ne);
+        e = allow_dyn_smem(short_kern, sm_short);
         if (e != cudaSuccess) return cuda_check(e, "k_interp_fx_short smem attribute");
         const int slot = timing_begin(p, "interp_fx_short");
-        const int64_t nb = (n + 32 * kFxsWarps - 1) / (32 * kFxsWarps);
-        k_interp_fx_short<<<(unsigned)std::min<int64_t>(nb, (int64_t)nsm * 3), 32 * kFxsWarps, sm_short, p->stream>>>(
-            p->geom, (const double2 *)maps, (const StencilRec64 *)b.rec, psi, b.perm, n, b.occ, kMean, tod);
+        const int64_t one = (int64_t)ctas * kFxsWarps;              // warps of one wave
+        const int64_t bs = std::max<int64_t>(4, std::min<int64_t>(32, (n + one - 1) / one));
+        const int64_t nb = (n + bs * kFxsWarps - 1) / (bs * kFxsWarps);
+        short_kern<<<(unsigned)std::min<int64_t>(nb, ctas), 32 * kFxsWarps, sm_short, p->stream>>>(
+            p->geom, (const double2 *)maps, (const StencilRec64 *)b.rec, psi, b.perm, n, (int)bs, b.occ, kMean, tod);
         timing_end(p, slot);
     }
     const int64_t nwarps = (n + chunk - 1) / chunk;
