@@ -189,7 +189,7 @@ constexpr int kRingGroup = 4;   // rings per sector of an FP32 G row (cluster fo
 // ------------------------------------------------------------------ in-place multi-ring form
 // One CTA transforms RG consecutive rings x KG consecutive k (TT = RG KG
 // transforms).  Shared memory holds units of TT values, unit e = element e of
-// every transform (t = ring-slot KG + k-slot), so each butterfly loads and
+// every transform (t = ring-slot KG + k-slot), so each FP32 butterfly loads and
 // stores whole units and reads its twiddles once for all TT transforms.  The
 // G reads of a CTA cover RG adjacent rings of one (k, m) row (G is ring-fastest)
 // and its cube writes KG adjacent k of one (ring, j) (the cube is k-fastest).
@@ -217,33 +217,56 @@ struct Swz {   // UB bytes per unit
 
 template <typename C, int R, int TT>
 __device__ __forceinline__ void dit_pass(C *x, int N, int Ns, const C *__restrict__ ptw) {
-    using Ut = FftUnit<C, TT>;
     using S = Swz<TT * (int)sizeof(C)>;
-    Ut *xu = reinterpret_cast<Ut *>(x);
     const bool p2 = (Ns & (Ns - 1)) == 0;
     const int lg = __ffs(Ns) - 1;
-    for (int b = threadIdx.x; b < N / R; b += blockDim.x) {
-        const int kk = p2 ? (b & (Ns - 1)) : b % Ns;
-        const int g = p2 ? (b >> lg) : b / Ns;
-        const int e0 = g * Ns * R + kk;
-        Ut u[R];
-#pragma unroll
-        for (int q = 0; q < R; ++q) u[q] = xu[S::at(e0 + q * Ns)];
-        C w[R];
-#pragma unroll
-        for (int q = 1; q < R; ++q) w[q] = Ns > 1 ? __ldg(ptw + (q - 1) * Ns + kk) : mk<C>(1.0, 0.0);
-#pragma unroll
-        for (int t = 0; t < TT; ++t) {
+    if constexpr (sizeof(C) == sizeof(double2)) {
+        // One butterfly of one transform a thread: with whole units a short ring's pass keeps
+        // a few half-empty warps (16 butterflies of radix 8 at nphi = 128) in long FP64 chains
+        // (K = 4, 127 x 128: 28.5 -> 13.8 us; K = 8, 256 x 512: 90 -> 72; K = 16, 1024 x 2048: 2.34 ->
+        // 2.28 ms).  FP32 keeps whole units: their accesses are 8 bytes wide otherwise.
+        for (int i = threadIdx.x; i < N / R * TT; i += blockDim.x) {
+            const int b = i / TT, t = i % TT;
+            const int kk = p2 ? (b & (Ns - 1)) : b % Ns;
+            const int g = p2 ? (b >> lg) : b / Ns;
+            const int e0 = g * Ns * R + kk;
             C v[R];
-            v[0] = u[0].v[t];
 #pragma unroll
-            for (int q = 1; q < R; ++q) v[q] = Ns > 1 ? mulc(u[q].v[t], w[q]) : u[q].v[t];
+            for (int q = 0; q < R; ++q) v[q] = x[S::at(e0 + q * Ns) * TT + t];
+            if (Ns > 1) {
+#pragma unroll
+                for (int q = 1; q < R; ++q) v[q] = mulc(v[q], __ldg(ptw + (q - 1) * Ns + kk));
+            }
             dft_small<C, true>(R, v);
 #pragma unroll
-            for (int q = 0; q < R; ++q) u[q].v[t] = v[q];
+            for (int q = 0; q < R; ++q) x[S::at(e0 + q * Ns) * TT + t] = v[q];
         }
+    } else {
+        using Ut = FftUnit<C, TT>;
+        Ut *xu = reinterpret_cast<Ut *>(x);
+        for (int b = threadIdx.x; b < N / R; b += blockDim.x) {
+            const int kk = p2 ? (b & (Ns - 1)) : b % Ns;
+            const int g = p2 ? (b >> lg) : b / Ns;
+            const int e0 = g * Ns * R + kk;
+            Ut u[R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) xu[S::at(e0 + q * Ns)] = u[q];
+            for (int q = 0; q < R; ++q) u[q] = xu[S::at(e0 + q * Ns)];
+            C w[R];
+#pragma unroll
+            for (int q = 1; q < R; ++q) w[q] = Ns > 1 ? __ldg(ptw + (q - 1) * Ns + kk) : mk<C>(1.0, 0.0);
+#pragma unroll
+            for (int t = 0; t < TT; ++t) {
+                C v[R];
+                v[0] = u[0].v[t];
+#pragma unroll
+                for (int q = 1; q < R; ++q) v[q] = Ns > 1 ? mulc(u[q].v[t], w[q]) : u[q].v[t];
+                dft_small<C, true>(R, v);
+#pragma unroll
+                for (int q = 0; q < R; ++q) u[q].v[t] = v[q];
+            }
+#pragma unroll
+            for (int q = 0; q < R; ++q) xu[S::at(e0 + q * Ns)] = u[q];
+        }
     }
 }
 
