@@ -13,44 +13,61 @@
 // Kernels (all FP64):
 //   k_orb_moments  one thread: the nine moments from b_lk, l <= 2
 //   k_orb_nodes    one thread per spline node: Eq. dipole_fast at that sample
-//   k_orb_spline   one warp per pointing period: second derivatives of the
-//                  natural cubic spline through the period's nodes
-//   k_orb_eval     one thread per sample: the spline between nodes, Eq.
+//   k_orb_spline   one CTA per pointing period: the cubics of the natural spline
+//                  through the period's nodes
+//   k_orb_eval     one thread per sample: the cubic between nodes, Eq.
 //                  dipole_fast after the last node (or everywhere when s = 1)
+// All are bound by the FP64 pipe (2 operations a clock and SM), so they keep its work
+// small: sines and cosines in 64-bit fixed point on the integer pipe (fx_sincos; absolute
+// error 2^-57, below the products' rounding), three multiply-adds a sample in the cubic.
+// 4e7 samples, s = 20 (nodes, spline, evaluation): 391, 155, 332 -> 154, 119, 274 us.
 //
-// The spline system M_{j-1} + 4 M_j + M_{j+1} = 6 (y_{j+1} - 2 y_j + y_{j-1}) / s^2
-// (M_0 = M_{n-1} = 0) is solved by the tridiagonal elimination
-//   dp_j = (rhs_j - dp_{j-1}) c_j,  M_j = dp_j - c_j M_{j+1},  c_j = 1 / (4 - c_{j-1}),
+// The spline system N_{j-1} + 4 N_j + N_{j+1} = y_{j+1} - 2 y_j + y_{j-1} (N = M s^2 / 6, M the
+// second derivatives, M_0 = M_{n-1} = 0) is solved by the tridiagonal elimination
+//   dp_j = (rhs_j - dp_{j-1}) c_j,  N_j = dp_j - c_j N_{j+1},  c_j = 1 / (4 - c_{j-1}),
 // whose pivots c_j reach their limit 2 - sqrt(3) (to the last bit) within
-// kOrbPivots rows.  Both sweeps are first-order recurrences with a factor of
-// magnitude c_j <= 0.268, so a run of rows started from zero differs from the
-// true values by that factor's powers times the true value before the run: a
-// warp stages 2048 rows in shared memory, gives each lane 64 consecutive rows,
-// runs them from zero (lane 0 from the true carry), and adds the carry of the
-// lane before it over the first kOrbFix rows (0.268^45 < 1e-25: the rest is
-// below rounding).
+// kOrbPivots rows.  Both sweeps are first-order recurrences d' = a - c d, affine in the value
+// before, so a thread runs kOrbRun rows from zero, the threads' maps (end value from zero, factor)
+// are combined by a scan, and each thread adds its rows' share of the value that enters it.
+// |c| <= 0.268: the factor of 64 rows (0.268^64 < 1e-36) is below any rounding, so the scan
+// combines 8 threads, and what enters a warp is the end value of the warp before.
 //
-// Between nodes the spline is w0 y_j + w1 y_{j+1} + w2 M_j + w3 M_{j+1} with
-// weights of r = t - j s only (B = r/s, A = 1 - B, w2 = (A^3 - A) s^2/6,
-// w3 = (B^3 - B) s^2/6), tabulated on the host: four FP64 operations a sample.
+// Between nodes j and j + 1 the spline is c0 + B (c1 + B (c2 + B c3)), B = r / s (a table),
+// r = t - j s, with c0 = y_j, c1 = y_{j+1} - y_j - (2 N_j + N_{j+1}), c2 = 3 N_j,
+// c3 = N_{j+1} - N_j.
 #include <cmath>
 
+#include "fxdigits.cuh"
 #include "sl_internal.cuh"
 
 namespace sl {
 
 constexpr int kOrbEvalPerThread = 8;   // samples per thread of k_orb_eval
-constexpr int kOrbRun = 64;            // rows per lane and sweep round of k_orb_spline
+constexpr int kOrbRun = 8;             // rows per thread and sweep round of k_orb_spline
 constexpr int kOrbPivots = 40;         // pivots tabulated; the last one is the limit
-constexpr int kOrbFix = 45;            // rows that take the carry of the lane before
 
 // Eq. dipole_fast at one sample.  beta' = Rz(-psi) Ry(-theta) Rz(-phi) beta.
-__device__ __forceinline__ double orb_value(const double *__restrict__ S, double T0, double q, double th,
-                                            double ph, double ps, const double *__restrict__ b) {
+// x 2^-62, x = 0 or |x| >= 1: the exponent lowered by integer arithmetic
+__device__ __forceinline__ double orb_q62(long long x) {
+    const double v = (double)x;
+    return x ? __hiloint2double(__double2hiint(v) - (62 << 20), __double2loint(v)) : 0.0;
+}
+__device__ __forceinline__ void orb_sincos(double x, const longlong2 *tab, double &s, double &c) {
+    long long fc, fs;
+    if (fx_sincos(x, tab, fc, fs)) {
+        s = orb_q62(fs);
+        c = orb_q62(fc);
+    } else {                                     // |x| >= 2^9 or not finite
+        sincos(x, &s, &c);
+    }
+}
+
+__device__ __forceinline__ double orb_value(const longlong2 *tab, const double *__restrict__ S, double T0, double q,
+                                            double th, double ph, double ps, const double *__restrict__ b) {
     double st, ct, sp, cp, ss, cs;
-    sincos(th, &st, &ct);
-    sincos(ph, &sp, &cp);
-    sincos(ps, &ss, &cs);
+    orb_sincos(th, tab, st, ct);
+    orb_sincos(ph, tab, sp, cp);
+    orb_sincos(ps, tab, ss, cs);
     const double u = cp * b[0] + sp * b[1];      // Rz(-phi)
     const double v = -sp * b[0] + cp * b[1];
     const double x1 = ct * u - st * b[2];        // Ry(-theta)
@@ -96,11 +113,13 @@ struct OrbArgs {
     const double *beta;       // [nper][3]
     const double *S;          // [9]
     const double *piv;        // [kOrbPivots] c_j (c_0 = 0); c_j = piv[kOrbPivots - 1] beyond
-    const double4_32a *w;     // [s + 1] spline weights (w0, w1, w2, w3) of r = 0 .. s
+    const double *frac;       // [s + 1] r / s
+    const longlong2 *tab;     // (cos, sin)(2 pi i / 256), Q62
     double T0, q;
     int64_t n, nper, nnodes;
     int s;
-    double *y, *M2;           // [nnodes] node values and spline second derivatives
+    double *y;                // [nnodes] node values
+    double4_32a *cub;         // [nnodes] cubics from each node on
     double *tod;
     int accumulate;
 };
@@ -119,97 +138,122 @@ __global__ void __launch_bounds__(256) k_orb_nodes(const OrbArgs a) {
          g += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = orb_find(a.noff, 0, a.nper, g);
         const int64_t i = a.start[p] + (int64_t)a.s * (g - a.noff[p]);
-        a.y[g] = orb_value(a.S, a.T0, a.q, a.theta[i], a.phi[i], a.psi[i], a.beta + 3 * p);
+        a.y[g] = orb_value(a.tab, a.S, a.T0, a.q, a.theta[i], a.phi[i], a.psi[i], a.beta + 3 * p);
     }
 }
 
-constexpr int kOrbWarps = 1;                      // periods (warps) per CTA of k_orb_spline (33 KB of static shared memory each)
-constexpr int kOrbRound = 32 * kOrbRun;           // rows per sweep round
-constexpr int kOrbPad = kOrbRound + kOrbRound / kOrbRun;
+constexpr int kOrbThreads = 256;
+constexpr int kOrbRound = kOrbThreads * kOrbRun;  // rows per sweep round
 
-// shared-memory slot of round row q: one pad slot per lane run, so that the 32
-// lanes (rows 64 l + i) fall on distinct bank pairs
-__device__ __forceinline__ int orb_pad(int q) { return q + (q >> 6); }
+// shared-memory slot of round row q: one pad slot per thread's run, so that the lanes'
+// rows (8 l + i) fall on distinct banks
+__device__ __forceinline__ int orb_pad(int q) { return q + (q >> 3); }
+constexpr int kOrbPad = kOrbRound + kOrbRound / kOrbRun + 2;
 
-// One warp per period: the two sweeps of the elimination in rounds of
-// kOrbRound rows staged in shared memory (coalesced loads and stores; each lane
-// runs its 64 rows from shared memory; see the header).
-__global__ void __launch_bounds__(32 * kOrbWarps) k_orb_spline(const OrbArgs a) {
-    __shared__ double s_piv[kOrbPivots];
-    __shared__ double s_y[kOrbWarps][kOrbRound + 2];
-    __shared__ double s_d[kOrbWarps][kOrbPad];
-    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
-    for (int j = threadIdx.x; j < kOrbPivots; j += blockDim.x) s_piv[j] = a.piv[j];
+// The value that enters this thread's rows, from every thread's (end value from zero A, factor F)
+// and the value that enters the round; ends[warp]: the warps' end values (ends[7]: the round's).
+__device__ __forceinline__ double orb_enter(double A, double F, double carry, double *ends) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const double pa = __shfl_up_sync(0xffffffffu, A, o), pf = __shfl_up_sync(0xffffffffu, F, o);
+        if (lane >= o) {
+            A = fma(F, pa, A);
+            F *= pf;
+        }
+    }
+    if (lane == 31) ends[warp] = A;
     __syncthreads();
-    const int64_t p = (int64_t)blockIdx.x * kOrbWarps + wq;
-    if (p >= a.nper) return;
+    const double in = warp ? ends[warp - 1] : carry;
+    const double pa = __shfl_up_sync(0xffffffffu, A, 1), pf = __shfl_up_sync(0xffffffffu, F, 1);
+    return lane ? fma(pf, in, pa) : in;
+}
+
+// One CTA per period: both sweeps in rounds of kOrbRound rows, values staged through shared
+// memory so that global accesses are coalesced.  The forward sweep's dp_j wait in the first
+// quarter of the period's cubics: cubic j (doubles 4 j .. 4 j + 3) replaces dp values of rows at
+// or above j, which the backward sweep has read by then.
+__global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
+    __shared__ double s_piv[kOrbPivots];
+    __shared__ double s_y[kOrbPad], s_d[kOrbPad];
+    __shared__ double s_end[2][kOrbThreads / 32];
+    for (int j = threadIdx.x; j < kOrbPivots; j += kOrbThreads) s_piv[j] = a.piv[j];
+    __syncthreads();
+    const int64_t p = blockIdx.x;
     const int64_t g0 = a.noff[p], M = a.noff[p + 1] - g0;
+    if (M < 2) return;
     const double *__restrict__ y = a.y + g0;
-    double *__restrict__ m2 = a.M2 + g0;
-    double *sy = s_y[wq], *sd = s_d[wq];
-    if (M < 3) {
-        for (int64_t j = lane; j < M; j += 32) m2[j] = 0.0;
-        return;
-    }
-    if (lane == 0) {
-        m2[0] = 0.0;
-        m2[M - 1] = 0.0;
-    }
+    double4_32a *cub = a.cub + g0;
+    double *dp = reinterpret_cast<double *>(cub);
     auto piv = [&](int64_t j) { return s_piv[j < kOrbPivots ? j : kOrbPivots - 1]; };
-    const double r6 = 6.0 / ((double)a.s * (double)a.s);
+    const int lo = threadIdx.x * kOrbRun;
+    int par = 0;                                     // s_end is used alternately: one barrier a round less
     // forward sweep over rows 1 .. M-2: dp_j = (rhs_j - dp_{j-1}) c_j, dp_0 = 0
     double carry = 0.0;
-    for (int64_t base = 1; base <= M - 2; base += kOrbRound) {
+    for (int64_t base = 1; base <= M - 2; base += kOrbRound, par ^= 1) {
         const int rows = (int)min((int64_t)kOrbRound, M - 1 - base);
-        for (int k = lane; k < rows + 2; k += 32) sy[k] = y[base - 1 + k];
-        __syncwarp();
-        for (int k = lane; k < rows; k += 32) sd[orb_pad(k)] = r6 * (sy[k + 2] - 2.0 * sy[k + 1] + sy[k]);
-        __syncwarp();
-        const int lo = lane * kOrbRun, hi = min(lo + kOrbRun, rows);
-        double d = lane == 0 ? carry : 0.0;
-        for (int q = lo; q < hi; ++q) {
-            d = (sd[orb_pad(q)] - d) * piv(base + q);
-            sd[orb_pad(q)] = d;
-        }
-        const double before = __shfl_up_sync(0xffffffffu, d, 1);
-        if (lane > 0 && lo < hi) {
-            double corr = before;
-            for (int q = lo; q < min(hi, lo + kOrbFix); ++q) {
-                corr *= -piv(base + q);
-                sd[orb_pad(q)] += corr;
+        for (int k = threadIdx.x; k < rows + 2; k += kOrbThreads) s_y[orb_pad(k)] = y[base - 1 + k];
+        __syncthreads();
+        double v[kOrbRun], d = 0.0, f = 1.0;
+#pragma unroll
+        for (int i = 0; i < kOrbRun; ++i)
+            if (lo + i < rows) {
+                const int k = lo + i;
+                const double c = piv(base + k);
+                d = (s_y[orb_pad(k + 2)] - 2.0 * s_y[orb_pad(k + 1)] + s_y[orb_pad(k)] - d) * c;
+                f *= -c;
+                v[i] = d;
             }
-        }
-        // the next round starts after lane 31's rows (its carry term there is
-        // below 0.268^64 of the value; with fewer rows the period has ended)
-        carry = __shfl_sync(0xffffffffu, d, 31);
-        __syncwarp();
-        for (int k = lane; k < rows; k += 32) m2[base + k] = sd[orb_pad(k)];
-        __syncwarp();
+        double in = orb_enter(d, f, carry, s_end[par]);
+        carry = s_end[par][kOrbThreads / 32 - 1];
+#pragma unroll
+        for (int i = 0; i < kOrbRun; ++i)
+            if (lo + i < rows) {
+                in *= -piv(base + lo + i);
+                s_d[orb_pad(lo + i)] = v[i] + in;
+            }
+        __syncthreads();
+        for (int k = threadIdx.x; k < rows; k += kOrbThreads) dp[base + k] = s_d[orb_pad(k)];
     }
-    // backward sweep: M_j = dp_j - c_j M_{j+1}, M_{M-1} = 0; round row q is j = top - q
+    __syncthreads();                                 // dp is read by other threads than wrote it
+    // backward sweep: N_j = dp_j - c_j N_{j+1}, N_{M-1} = 0; round row q is j = top - q, then the
+    // cubics of nodes top .. top - rows + 1, from N_j and N_{j+1}
     carry = 0.0;
-    for (int64_t top = M - 2; top >= 1; top -= kOrbRound) {
+    double above = 0.0;                              // N of the row above the round
+    for (int64_t top = M - 2; top >= 1; top -= kOrbRound, par ^= 1) {
         const int rows = (int)min((int64_t)kOrbRound, top);
-        for (int k = lane; k < rows; k += 32) sd[orb_pad(k)] = m2[top - k];
-        __syncwarp();
-        const int lo = lane * kOrbRun, hi = min(lo + kOrbRun, rows);
-        double m = lane == 0 ? carry : 0.0;
-        for (int q = lo; q < hi; ++q) {
-            m = sd[orb_pad(q)] - piv(top - q) * m;
-            sd[orb_pad(q)] = m;
-        }
-        const double above = __shfl_up_sync(0xffffffffu, m, 1);
-        if (lane > 0 && lo < hi) {
-            double corr = above;
-            for (int q = lo; q < min(hi, lo + kOrbFix); ++q) {
-                corr *= -piv(top - q);
-                sd[orb_pad(q)] += corr;
+        for (int k = threadIdx.x; k < rows; k += kOrbThreads) s_d[orb_pad(k)] = dp[top - k];
+        for (int k = threadIdx.x; k < rows + 1; k += kOrbThreads) s_y[orb_pad(k)] = y[top + 1 - k];
+        __syncthreads();
+        double v[kOrbRun], m = 0.0, f = 1.0;
+#pragma unroll
+        for (int i = 0; i < kOrbRun; ++i)
+            if (lo + i < rows) {
+                const double c = piv(top - lo - i);
+                m = s_d[orb_pad(lo + i)] - c * m;
+                f *= -c;
+                v[i] = m;
             }
+        double in = orb_enter(m, f, carry, s_end[par]);
+        carry = s_end[par][kOrbThreads / 32 - 1];
+#pragma unroll
+        for (int i = 0; i < kOrbRun; ++i)
+            if (lo + i < rows) {
+                in *= -piv(top - lo - i);
+                s_d[orb_pad(lo + i)] = v[i] + in;
+            }
+        __syncthreads();
+        for (int k = threadIdx.x; k < rows; k += kOrbThreads) {
+            const double m0 = s_d[orb_pad(k)], m1 = k ? s_d[orb_pad(k - 1)] : above;
+            const double y0 = s_y[orb_pad(k + 1)], y1 = s_y[orb_pad(k)];
+            cub[top - k] = make_double4_32a(y0, (y1 - y0) - fma(2.0, m0, m1), 3.0 * m0, m1 - m0);
         }
-        carry = __shfl_sync(0xffffffffu, m, 31);
-        __syncwarp();
-        for (int k = lane; k < rows; k += 32) m2[top - k] = sd[orb_pad(k)];
-        __syncwarp();
+        above = s_d[orb_pad(rows - 1)];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double m1 = above;                     // node 0: N_0 = 0, N_1 (0 when there are two nodes)
+        cub[0] = make_double4_32a(y[0], (y[1] - y[0]) - m1, 0.0, m1);
     }
 }
 
@@ -243,15 +287,15 @@ __global__ void __launch_bounds__(256) k_orb_eval(const OrbArgs a) {
             } else {
                 const unsigned j = jt < M - 1 ? jt : M - 2;
                 if (SL_GUARD(g0 + j + 1 < a.nnodes && t - j * su <= su, 0x501u)) {
-                    const double4_32a w = a.w[t - j * su];         // r = t - j s (s at the last node)
-                    const double *yy = a.y + g0 + j, *mm = a.M2 + g0 + j;
-                    val = w.x * yy[0] + w.y * yy[1] + w.z * mm[0] + w.w * mm[1];
+                    const double B = __ldg(a.frac + (t - j * su));      // r = t - j s (s at the last node)
+                    const double4_32a c = a.cub[g0 + j];
+                    val = fma(B, fma(B, fma(B, c.w, c.z), c.y), c.x);
                 } else {
                     val = 0.0;
                 }
             }
         }
-        if (exact) val = orb_value(a.S, a.T0, a.q, a.theta[i], a.phi[i], a.psi[i], a.beta + 3 * p);
+        if (exact) val = orb_value(a.tab, a.S, a.T0, a.q, a.theta[i], a.phi[i], a.psi[i], a.beta + 3 * p);
         a.tod[i] = a.accumulate ? a.tod[i] + val : val;
     }
 }
@@ -271,7 +315,8 @@ sl_status launch_orbital(sl_plan *p, const OrbLaunch &o) {
     a.beta = o.beta;
     a.S = o.S;
     a.piv = o.piv;
-    a.w = reinterpret_cast<const double4_32a *>(o.w);
+    a.frac = o.frac;
+    a.tab = p->geom.phase_tab;
     a.T0 = o.T0;
     a.q = o.q;
     a.n = o.n;
@@ -279,7 +324,7 @@ sl_status launch_orbital(sl_plan *p, const OrbLaunch &o) {
     a.nnodes = o.nnodes;
     a.s = o.s;
     a.y = o.y;
-    a.M2 = o.M2;
+    a.cub = reinterpret_cast<double4_32a *>(o.cub);
     a.tod = o.tod;
     a.accumulate = o.accumulate;
     int slot;
@@ -291,7 +336,7 @@ sl_status launch_orbital(sl_plan *p, const OrbLaunch &o) {
         sl_status st = cuda_check(cudaGetLastError(), "k_orb_nodes launch");
         if (st != SL_OK) return st;
         slot = timing_begin(p, "orb_spline");
-        k_orb_spline<<<(unsigned)((a.nper + kOrbWarps - 1) / kOrbWarps), 32 * kOrbWarps, 0, p->stream>>>(a);
+        k_orb_spline<<<(unsigned)a.nper, kOrbThreads, 0, p->stream>>>(a);
         timing_end(p, slot);
         if ((st = cuda_check(cudaGetLastError(), "k_orb_spline launch")) != SL_OK) return st;
     }

@@ -1054,12 +1054,11 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     // the pinned staging buffer is reused: wait until the previous upload has left it
     if (p->orb_ev && (st = cuda_check(cudaEventSynchronize(p->orb_ev), "orbital staging")) != SL_OK) return st;
     // host tables: [start | noff] as int64, then beta [nper][3], the elimination
-    // pivots c_j = 1 / (4 - c_{j-1}) (c_0 = 0) and the spline weights of the
-    // positions r = 0 .. s between two nodes (B = r/s, A = 1 - B)
+    // pivots c_j = 1 / (4 - c_{j-1}) (c_0 = 0) and the positions r / s, r = 0 .. s, between
+    // two nodes
     constexpr int kPiv = 40;
-    const size_t nw = 4 * ((size_t)subsample + 1);
-    // layout [weights | pivots | start | noff | beta]: the weights (read as 32-byte
-    // vectors) first, at a 32-byte aligned offset of the scratch
+    const size_t nw = (size_t)subsample + 1;
+    // layout [positions | pivots | start | noff | beta]
     const size_t tab_bytes = (nw + kPiv + 2 * (size_t)(nper + 1) + 3 * (size_t)nper) * sizeof(int64_t);
     if (tab_bytes > p->h_orb_bytes) {
         if (p->h_orb) cudaFreeHost(p->h_orb);
@@ -1080,14 +1079,7 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     double *bet = reinterpret_cast<double *>(noff + (nper + 1));
     piv[0] = 0.0;
     for (int j = 1; j < kPiv; ++j) piv[j] = 1.0 / (4.0 - piv[j - 1]);
-    const double sd = (double)subsample, h2 = sd * sd / 6.0;
-    for (int r = 0; r <= subsample; ++r) {
-        const double B = (double)r / sd, A = 1.0 - B;
-        wt[4 * r + 0] = A;
-        wt[4 * r + 1] = B;
-        wt[4 * r + 2] = (A * A * A - A) * h2;
-        wt[4 * r + 3] = (B * B * B - B) * h2;
-    }
+    for (int r = 0; r <= subsample; ++r) wt[r] = (double)r / (double)subsample;
     noff[0] = 0;
     for (int64_t k = 0; k < nper; ++k) {
         const int64_t np = period_start[k + 1] - period_start[k];
@@ -1103,11 +1095,13 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     }
     start[nper] = n;
     const int64_t nnodes = noff[nper];
-    const size_t need = kOrbS * sizeof(double) + tab_bytes + 2 * (size_t)nnodes * sizeof(double);
+    // scratch [moments | tables | cubics (32-byte vectors) | node values]
+    const size_t cub_off = (kOrbS * sizeof(double) + tab_bytes + 31) / 32 * 32;
+    const size_t need = cub_off + 5 * (size_t)nnodes * sizeof(double);
     if ((st = orb_scratch(p, need)) != SL_OK) return st;
     char *base = reinterpret_cast<char *>(p->d_orb);
     int64_t *d_tab = reinterpret_cast<int64_t *>(base + kOrbS * sizeof(double));
-    double *d_nodes = reinterpret_cast<double *>(base + kOrbS * sizeof(double) + tab_bytes);
+    double *d_nodes = reinterpret_cast<double *>(base + cub_off);
     if ((st = cuda_check(cudaMemcpyAsync(d_tab, p->h_orb, tab_bytes, cudaMemcpyHostToDevice, p->stream),
                          "orbital tables")) != SL_OK)
         return st;
@@ -1117,8 +1111,8 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     o.theta = theta;
     o.phi = phi;
     o.psi = psi;
-    o.w = reinterpret_cast<const double *>(d_tab);
-    o.piv = o.w + nw;
+    o.frac = reinterpret_cast<const double *>(d_tab);
+    o.piv = o.frac + nw;
     o.start = d_tab + nw + kPiv;
     o.noff = o.start + (nper + 1);
     o.beta = reinterpret_cast<const double *>(o.noff + (nper + 1));
@@ -1129,8 +1123,8 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     o.nper = nper;
     o.nnodes = nnodes;
     o.s = subsample;
-    o.y = d_nodes;
-    o.M2 = d_nodes + nnodes;
+    o.cub = d_nodes;
+    o.y = d_nodes + 4 * nnodes;
     o.tod = tod;
     o.accumulate = accumulate != 0;
     return launch_orbital(p, o);

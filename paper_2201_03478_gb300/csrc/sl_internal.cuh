@@ -383,11 +383,11 @@ struct OrbLaunch {
     const int64_t *start, *noff;
     const double *beta, *S;
     const double *piv;       // elimination pivots c_1 .. c_39 (c_0 = 0), the last one the limit
-    const double *w;         // [s][4] spline weights per position between nodes
+    const double *frac;      // [s + 1] position between nodes r / s
     double T0, q;
     int64_t n, nper, nnodes;
     int s;
-    double *y, *M2, *tod;
+    double *y, *cub, *tod;   // cub: [nnodes][4], 32-byte aligned
     int accumulate;
 };
 sl_status launch_orb_moments(sl_plan *p, const double *beam, double *S);
