@@ -346,18 +346,12 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                                 }
                             }
                         }
-                        if (kOne) {                 // the next cell of this stretch
-                            const unsigned here = __shfl_sync(0xffffffffu, mycell, r1 & 31);
-                            const unsigned ahead = __shfl_sync(0xffffffffu, r_next.cell, 0);
-                            if (r1 < cnt) fx_fetch<P>(g, maps, here, 0, 0, gr, q4, lane, raw);
-                            else if (t0 + 32 < wlast && ahead != cell) fx_fetch<P>(g, maps, ahead, 0, 0, gr, q4, lane, raw);
-                        }
-                    } else if (kOne && r1 == cnt && t0 + 32 < wlast) {
-                        // the operand is kept past this batch's end: fetch the next batch's first cell
+                    }
+                    if (kOne) {                     // the stretch's next cell, at one place (code size)
+                        const unsigned here = __shfl_sync(0xffffffffu, mycell, r1 & 31);
                         const unsigned ahead = __shfl_sync(0xffffffffu, r_next.cell, 0);
-                        if (ahead != cell) fx_fetch<P>(g, maps, ahead, 0, 0, gr, q4, lane, raw);
-                    } else if (kOne && r1 < cnt) {
-                        fx_fetch<P>(g, maps, __shfl_sync(0xffffffffu, mycell, r1 & 31), 0, 0, gr, q4, lane, raw);
+                        if (r1 < cnt || (t0 + 32 < wlast && ahead != cell))
+                            fx_fetch<P>(g, maps, r1 < cnt ? here : ahead, 0, 0, gr, q4, lane, raw);
                     }
                     const bool mine_in_run = lane >= r0 && lane < r1;
                     if (a_ef == 2047) {             // uniform over the warp: no row tile is summed
