@@ -227,8 +227,8 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
     meas = {"fp64": alu.get("fp64"), "fp32": alu.get("fp32")}
     kernels = [
         (lc_name,
-         # FP64: digit products executed, 60 m16n8k8 per 32 recurrences and 8 l
-         {"fp64": 60 * 2.0 * 16 * 8 * 8 / 256 * lsteps, "fp32": fl_lc, "df64": DF_LC_INST_PER_STEP * lsteps,
+         # FP64: digit products executed, 30 m16n8k8 per 32 recurrences and 8 l
+         {"fp64": 30 * 2.0 * 16 * 8 * 8 / 256 * lsteps, "fp32": fl_lc, "df64": DF_LC_INST_PER_STEP * lsteps,
           # tensor work executed: 3 TF32 products x 2 flops x 16 columns (4 used, one sky)
           "tf32x3": 3 * 2.0 * 16 * lsteps}[prec],
          {"fp64": "fp16", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "tf32"}[prec]),
@@ -283,21 +283,21 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
 
 
 def adjoint_roofs(stats, plan, K, n, alu, traffic_ok=True):
-    """FP64 adjoint kernels: the interpolation transpose does the forward's
-    multiply-adds per sample (4 p^2 (K+1) + 10 flops), the contraction transpose
-    11 flops per (ring, m, k, sign, l) step of the forward's volume."""
+    """Adjoint kernels in fixed point on the tensor cores: the digit products of full
+    tiles (interpolation transpose: 6 + 27 ceil(K/4) m16n8k16 per 16 samples of a cell;
+    contraction transpose: 30 m16n8k16 per 32 recurrences and 16 l)."""
     lsteps = float(plan.sizes()["lsteps"])
+    peak = float(measured_peaks().get("bf16_tflops", 1900.0))
     out = {}
-    for name, work in (("interp_adj", float(n) * (4.0 * 16 * (K + 1) + 10.0)), ("lcontract_adj", 11.0 * lsteps)):
+    for name, work in (("interp_adj_fx", float(n) / 16 * (6 + 27 * ((K + 3) // 4)) * 2.0 * 16 * 8 * 16),
+                       ("lcontract_adj_fx", 30 * 2.0 * 16 * 8 * 16 / 512 * lsteps)):
         if name in stats and stats[name][0] > 0:
             avg_ms = stats[name][1] / stats[name][0]
             ach = work / (avg_ms / 1e3) / 1e12
-            out[name] = {"bound": "alu", "achieved": round(ach, 4), "peak": round(PEAK_FP64_TFLOPS, 4),
-                         "unit": "TFLOP/s", "frac": round(ach / PEAK_FP64_TFLOPS, 4), "avg_ms": round(avg_ms, 4),
+            out[name] = {"bound": "tensor", "achieved": round(ach, 4), "peak": round(peak, 4),
+                         "unit": "TFLOP/s", "frac": round(ach / peak, 4), "avg_ms": round(avg_ms, 4),
                          "flops_per_launch": work, "traffic": TRAFFIC.get((name, "fp64")) if traffic_ok else None,
-                         "peak_note": "derived: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz"}
-            if alu.get("fp64"):
-                out[name]["frac_of_measured_alu_peak"] = round(ach / alu["fp64"], 4)
+                         "peak_note": "measured bf16 burst (MEASURED_PEAKS.json); digit products of full tiles"}
     return out
 
 
@@ -796,14 +796,10 @@ def multisky_arm(args):
 TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum per launch, LFI-like workload, 1e8 pointings
     # (profiles/launches_lfi_{fp64,fp32,df64}.txt; single-pass ncu metrics of the current kernels)
-    ("lcontract_f64", "fp64"): 673.9e6 + 516.4e6,
-    ("interp_f64", "fp64"): 15153.3e6 + 1911.1e6,
     ("lcontract_f32", "fp32"): 370.3e6 + 233.7e6,
     ("interp_f32", "fp32"): 7086.2e6 + 2115.9e6,
     ("lcontract_df", "df64"): 672.3e6 + 511.3e6,
     ("interp_df", "df64"): 22934.1e6 + 2736.6e6,
-    ("interp_adj", "fp64"): 18463.7e6 + 385.5e6,
-    ("lcontract_adj", "fp64"): 1507.2e6 + 285.3e6,
 }
 
 

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(1024) k_scan_local(int64_t n, unsigned *__rest
 // earlier totals itself (nb^2 / 2 words from L2, 0.5 MB at 1024 x 2048 cells): a scan of them by
 // one CTA in between, and of the tiles' chunks by another, cost the small and sparse sorts two
 // launches, and with the tiles' strided words more than the rest of the scan (1500 x 3000
-// cells: 17 + 5 + 12 + 4 + 66 us; both kernels now 17 us at 1024 x 2048, 24 before).
+// cells: 17 + 5 + 12 + 4 + 66 us, now 10 + 11 + 37).
 __global__ void __launch_bounds__(1024) k_scan_add(int64_t n, unsigned *__restrict__ data, const unsigned *__restrict__ bsum,
                                                     const unsigned *__restrict__ nz, unsigned *__restrict__ cursor,
                                                     unsigned *__restrict__ occ) {
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(kAggThreads) k_scatter_agg(int64_t n, int64_t 
 }
 
 // chunk_off[t] = sum over the tiles before t of ceil(#samples / kChunk), chunk_off[ntiles] = total.
-// One CTA per 1024 tiles, which also sums the chunks of the tiles before its own (up to 64
-// strided rounds of independent loads at the largest grids).
+// One CTA per 1024 tiles, which also sums the chunks of the tiles before its own (37 us at 1500 x
+// 3000 cells, bound by its strided reads; the counts and a single CTA's scan took 4 + 66).
 __global__ void __launch_bounds__(1024) k_tile_chunks(int ntiles, int ncell, const unsigned *__restrict__ start,
                                                        unsigned *__restrict__ chunk_off) {
     auto chunks = [&](int t) {
