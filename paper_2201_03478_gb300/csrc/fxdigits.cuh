@@ -45,6 +45,13 @@ __device__ __forceinline__ long long fx_mulhi(long long a, long long b) {
 }
 // a b for Q62 operands (|a|, |b| <= 1): Q62, at most 2^-59 off
 __device__ __forceinline__ long long fx_mul(long long a, long long b) { return fx_mulhi(a, b) << 2; }
+// the same rounded to nearest, without the truncation's bias (zero stays zero): at most 2^-61 off
+__device__ __forceinline__ long long fx_mul_rn(long long a, long long b) {
+    const int al = (int)a, bl = (int)b;
+    const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31), bh = (int)(b >> 32) + (int)((unsigned)bl >> 31);
+    const long long m = (long long)ah * bl + (long long)bh * al;
+    return (long long)ah * bh * 4 + ((m + (1ll << 29)) >> 30);
+}
 
 // digit pairs (a's digit in the low half, b's in the high half) of two Q62 values:
 // the 9-bit field u goes into the mantissa of FP16 1024 + u, minus 1280
@@ -53,7 +60,10 @@ __device__ __forceinline__ uint32_t fx_field(uint32_t a, uint32_t b, uint32_t ma
     const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&u), __halves2half2(__ushort_as_half(0x6500), __ushort_as_half(0x6500)));
     return *reinterpret_cast<const uint32_t *>(&h);
 }
-__device__ __forceinline__ void fx_digits(long long a, long long b, uint32_t d[kFxDig]) {
+// N = 6: rounded to 53 fraction bits; N = 7: a seventh digit 2^-62 takes what the six leave over (exact)
+template <int N>
+__device__ __forceinline__ void fx_digits(long long a, long long b, uint32_t (&d)[N]) {
+    static_assert(N == kFxDig || N == kFxDig + 1, "six digits or seven");
     const unsigned long long ya = (unsigned long long)a + kFxBias, yb = (unsigned long long)b + kFxBias;
     const uint32_t ah = (uint32_t)(ya >> 32), al = (uint32_t)ya, bh = (uint32_t)(yb >> 32), bl = (uint32_t)yb;
     d[0] = fx_field(ah >> 22, bh >> 22, 0x03ff03ffu);
@@ -62,6 +72,7 @@ __device__ __forceinline__ void fx_digits(long long a, long long b, uint32_t d[k
     d[3] = fx_field(__funnelshift_r(al, ah, 27), __funnelshift_r(bl, bh, 27), 0x01ff01ffu);
     d[4] = fx_field(al >> 18, bl >> 18, 0x01ff01ffu);
     d[5] = fx_field(al >> 9, bl >> 9, 0x01ff01ffu);
+    if constexpr (N > kFxDig) d[6] = fx_field(al, bl, 0x01ff01ffu);
 }
 
 // x 2^(62 - e) (truncated toward zero below 2^-62) for |x| < 2^e, e = ef - 1022, by
@@ -110,6 +121,20 @@ __device__ __forceinline__ long long fx_combine(const float (&a)[kFxSums]) {
     x += (long long)__float2int_rn(a[6]) * 512ll;
     x += (long long)__float2int_rn(a[5]) * 262144ll;
     long long v = x >> 22;
+    v += (long long)__float2int_rn(a[4]) * 32ll;
+    v += (long long)__float2int_rn(a[3]) * 16384ll;
+    v += (long long)__float2int_rn(a[2]) * 8388608ll;
+    v += (long long)((unsigned long long)(uint32_t)(__float2int_rn(a[1]) + (__float2int_rn(a[0]) << 9)) << 32);
+    return v;
+}
+// x 2^-n rounded to nearest, ties to even
+__device__ __forceinline__ long long fx_shift_even(long long x, int n) {
+    return n > 0 ? (x + ((1ll << (n - 1)) - 1) + ((x >> n) & 1)) >> n : x;
+}
+// the same from the digit sums of orders 0 to 6 alone, rounded to even: with one factor 1 a 32nd
+// of the sums are ties
+__device__ __forceinline__ long long fx_combine(const float (&a)[kFxSums - 1]) {
+    long long v = fx_shift_even((long long)__float2int_rn(a[6]) + (long long)__float2int_rn(a[5]) * 512ll, 13);
     v += (long long)__float2int_rn(a[4]) * 32ll;
     v += (long long)__float2int_rn(a[3]) * 16384ll;
     v += (long long)__float2int_rn(a[2]) * 8388608ll;

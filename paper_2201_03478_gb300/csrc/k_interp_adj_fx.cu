@@ -39,11 +39,12 @@ namespace sl {
 
 constexpr int kFaWarps = 4;
 constexpr int kFaRow = 20;         // words per row of 32 samples (padded: fragment rows in distinct banks)
+constexpr int kFaDig = 7;          // digits of y w (the phases have six); products of orders 0 to 6
 constexpr int kFaEmpty = -4096;    // exponent of sums that are all zero
 constexpr int kFaChunk = 512;      // longest stretch of a warp: keeps the 64-bit sums in range
 
 struct FaWarp {                    // one warp's shared memory; sums follow (fa_sums)
-    uint32_t a[6][16][kFaRow];     // digits of y w: [digit][4 row + column mod 4][sample pair]
+    uint32_t a[kFaDig][16][kFaRow];     // digits of y w: [digit][4 row + column mod 4][sample pair]
     uint32_t e[6][8][kFaRow];      // digits of the phases of 4 orders: [digit][2 order + part][sample pair]
 };
 // bytes per warp with the sums of order 0 (2 rows) and of blocks of 4 orders (2 rows x re, im)
@@ -197,25 +198,26 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
             }
             const unsigned later = lane < 31 ? heads & (0xfffffffeu << lane) : 0u;
             ey = __shfl_sync(0xffffffffu, ey, (later ? __ffs(later) - 1 : cnt) - 1);
-            // y w 2^(61 - e), e = ey - 1022; |w| < 2.  Sums over thousands of samples would show a
-            // bias: the first product's truncation (4 units) is centred, the second's is centred by
-            // the digits' rounding, and the sums below round ties to even.
+            // y w 2^(61 - e), e = ey - 1022; |w| < 2.  Sums over thousands of samples show a bias, so
+            // both products are rounded to nearest, and what is shifted below rounds ties to even.  All of
+            // its 62 bits enter the seven digits (1e7 uniform samples on 127 x 128 cells, cube against long
+            // double: 5.9e-16; six digits, 2^-53 of twice the run's largest |y|: 16e-16; FP64: 6.7e-16).
             const long long yq = use ? fx_from_double(y, ey) >> 1 : 0;
             __half *arow = reinterpret_cast<__half *>(&W.a[0][0][lane >> 1]) + (lane & 1);
 #pragma unroll 1
             for (int a = 0; a < 4; ++a) {
-                const long long ya = fx_mul(yq, lwt[0]) + 2;
+                const long long ya = fx_mul_rn(yq, lwt[0]);
                 lwt[0] = lwt[1];
                 lwt[1] = lwt[2];
                 lwt[2] = lwt[3];
 #pragma unroll
                 for (int b = 0; b < 4; b += 2) {
-                    uint32_t d[kFxDig];
-                    fx_digits(fx_mul(ya, lwp[b]), fx_mul(ya, lwp[b + 1]), d);
+                    uint32_t d[kFaDig];
+                    fx_digits(fx_mul_rn(ya, lwp[b]), fx_mul_rn(ya, lwp[b + 1]), d);
                     __half *o0 = arow + (4 * a + ((j - 1 + b) & 3)) * (2 * kFaRow);
                     __half *o1 = arow + (4 * a + ((j + b) & 3)) * (2 * kFaRow);
 #pragma unroll
-                    for (int u = 0; u < kFxDig; ++u) {
+                    for (int u = 0; u < kFaDig; ++u) {
                         const __half2 h = *reinterpret_cast<const __half2 *>(&d[u]);
                         o0[u * (16 * 2 * kFaRow)] = __low2half(h);
                         o1[u * (16 * 2 * kFaRow)] = __high2half(h);
@@ -281,28 +283,27 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                 int shift = 3;
                 if (en > e) {
                     if (e != kFaEmpty) {
-                        const int d = min(en - e, 63);
-                        for (int q = 0; q < nv; ++q) v[32 * q] = (v[32 * q] + ((1ll << d) >> 1)) >> d;
+                        const int d = en - e;
+                        for (int q = 0; q < nv; ++q) v[32 * q] = d > 61 ? 0 : fx_shift_even(v[32 * q], d);
                     }
                     e = en;
                 } else {
                     shift = min(3 + e - en, 62);
                 }
-                const long long half = (1ll << (shift - 1)) - 1;
-                float acc[4][kFxSums];
+                float acc[4][kFaDig];
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
 #pragma unroll
-                    for (int u = 0; u < kFxSums; ++u) acc[q][u] = 0.f;
+                    for (int u = 0; u < kFaDig; ++u) acc[q][u] = 0.f;
                 // the run's samples within each half of the batch
 #pragma unroll 1
                 for (int t = r0 >> 4; t <= (r1 - 1) >> 4; ++t) {
                     const int p0 = 16 * t + 2 * q4, p1 = p0 + 8;
                     const uint32_t m0 = (p0 >= r0 && p0 < r1 ? 0xffffu : 0u) | (p0 + 1 >= r0 && p0 + 1 < r1 ? 0xffff0000u : 0u);
                     const uint32_t m1 = (p1 >= r0 && p1 < r1 ? 0xffffu : 0u) | (p1 + 1 >= r0 && p1 + 1 < r1 ? 0xffff0000u : 0u);
-                    uint32_t ad[kFxDig][4];
+                    uint32_t ad[kFaDig][4];
 #pragma unroll
-                    for (int u = 0; u < kFxDig; ++u) {
+                    for (int u = 0; u < kFaDig; ++u) {
                         ad[u][0] = W.a[u][gr][8 * t + q4] & m0;
                         ad[u][1] = W.a[u][gr + 8][8 * t + q4] & m0;
                         ad[u][2] = W.a[u][gr][8 * t + q4 + 4] & m1;
@@ -311,15 +312,15 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                     if (b < 0) {
                         const uint32_t one = gr == 0 ? 0x5c005c00u : 0u;
 #pragma unroll
-                        for (int u = 0; u < kFxDig; ++u)
+                        for (int u = 0; u < kFaDig; ++u)
                             mma_f16(acc[0][u], acc[1][u], acc[2][u], acc[3][u], ad[u], one, one);
                     } else {
 #pragma unroll
                         for (int w = 0; w < kFxDig; ++w) {
                             const uint32_t b0 = W.e[w][gr][8 * t + q4], b1 = W.e[w][gr][8 * t + q4 + 4];
 #pragma unroll
-                            for (int u = 0; u < kFxDig; ++u)
-                                if (u < 3 || w < 3)
+                            for (int u = 0; u < kFaDig; ++u)
+                                if (u + w < kFaDig)
                                     mma_f16(acc[0][u + w], acc[1][u + w], acc[2][u + w], acc[3][u + w], ad[u], b0, b1);
                         }
                     }
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                 // (row gr, re), (row gr, im), (row gr + 8, re), (row gr + 8, im); order 0: re only
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const long long x = fx_combine(acc[q]), c = (x + half + ((x >> shift) & 1)) >> shift;
+                    const long long c = fx_shift_even(fx_combine(acc[q]), shift);
                     if (b >= 0) v[32 * q] += c;
                     else if (!(q & 1)) v[16 * q] += c;
                 }
