@@ -43,6 +43,13 @@ __device__ __forceinline__ long long fx_mulhi(long long a, long long b) {
     const long long m = (long long)ah * bl + (long long)bh * al;
     return (long long)ah * bh + (m >> 32);
 }
+// the same rounded to nearest; |a| < 2^62.6 with |b| <= 1.5 x 2^62 is in range too
+__device__ __forceinline__ long long fx_mulhi_rn(long long a, long long b) {
+    const int al = (int)a, bl = (int)b;
+    const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31), bh = (int)(b >> 32) + (int)((unsigned)bl >> 31);
+    const long long m = (long long)ah * bl + ((long long)bh * al + (1ll << 31));
+    return (long long)ah * bh + (m >> 32);
+}
 // a b for Q62 operands (|a|, |b| <= 1): Q62, at most 2^-59 off
 __device__ __forceinline__ long long fx_mul(long long a, long long b) { return fx_mulhi(a, b) << 2; }
 // the same rounded to nearest, without the truncation's bias (zero stays zero): at most 2^-61 off
@@ -53,20 +60,25 @@ __device__ __forceinline__ long long fx_mul_rn(long long a, long long b) {
     return (long long)ah * bh * 4 + ((m + (1ll << 29)) >> 30);
 }
 
+// Digits for operands of twice the range: x in (-2 + 2^-7, 2 - 2^-7), X = x 2^62, d_0 within
+// +-512, which FP16 and the sums above still hold (32 x (5 x 2^16 + 2^17) < 2^24).
+constexpr unsigned long long kFxBiasWide = kFxBias + (1ull << 62);
+
 // digit pairs (a's digit in the low half, b's in the high half) of two Q62 values:
 // the 9-bit field u goes into the mantissa of FP16 1024 + u, minus 1280
-__device__ __forceinline__ uint32_t fx_field(uint32_t a, uint32_t b, uint32_t mask) {
+__device__ __forceinline__ uint32_t fx_field(uint32_t a, uint32_t b, uint32_t mask, unsigned short offset = 0x6500) {
     const uint32_t u = (__byte_perm(a, b, 0x5410) & mask) | 0x64006400u;
-    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&u), __halves2half2(__ushort_as_half(0x6500), __ushort_as_half(0x6500)));
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&u), __halves2half2(__ushort_as_half(offset), __ushort_as_half(offset)));
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 // N = 6: rounded to 53 fraction bits; N = 7: a seventh digit 2^-62 takes what the six leave over (exact)
-template <int N>
+template <bool WIDE = false, int N>
 __device__ __forceinline__ void fx_digits(long long a, long long b, uint32_t (&d)[N]) {
     static_assert(N == kFxDig || N == kFxDig + 1, "six digits or seven");
-    const unsigned long long ya = (unsigned long long)a + kFxBias, yb = (unsigned long long)b + kFxBias;
+    constexpr unsigned long long kBias = WIDE ? kFxBiasWide : kFxBias;
+    const unsigned long long ya = (unsigned long long)a + kBias, yb = (unsigned long long)b + kBias;
     const uint32_t ah = (uint32_t)(ya >> 32), al = (uint32_t)ya, bh = (uint32_t)(yb >> 32), bl = (uint32_t)yb;
-    d[0] = fx_field(ah >> 22, bh >> 22, 0x03ff03ffu);
+    d[0] = fx_field(ah >> 22, bh >> 22, 0x03ff03ffu, WIDE ? 0x6600 : 0x6500);   // minus 1536 or 1280
     d[1] = fx_field(ah >> 13, bh >> 13, 0x01ff01ffu);
     d[2] = fx_field(ah >> 4, bh >> 4, 0x01ff01ffu);
     d[3] = fx_field(__funnelshift_r(al, ah, 27), __funnelshift_r(bl, bh, 27), 0x01ff01ffu);
@@ -75,14 +87,16 @@ __device__ __forceinline__ void fx_digits(long long a, long long b, uint32_t (&d
     if constexpr (N > kFxDig) d[6] = fx_field(al, bl, 0x01ff01ffu);
 }
 
-// x 2^(62 - e) (truncated toward zero below 2^-62) for |x| < 2^e, e = ef - 1022, by
+// x 2^(Q - e) (truncated toward zero below the unit) for |x| < 2^e, e = ef - 1022, by
 // its bits; ef: the largest biased exponent among the values sharing the scale,
 // 64 <= ef < 2047.  Values 2^64 times smaller than the scale give 0.
+template <int Q = 62>
 __device__ __forceinline__ long long fx_from_double(double x, int ef) {
+    static_assert(Q == 62 || Q == 63, "sign bit left");
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int ex = (int)(b >> 52) & 0x7ff;
     const int sh = min(ef - ex, 63);
-    const unsigned long long m = (((b & ((1ull << 52) - 1)) | (1ull << 52)) << 9) >> sh;
+    const unsigned long long m = (((b & ((1ull << 52) - 1)) | (1ull << 52)) << (Q - 53)) >> sh;
     const long long sg = (long long)b >> 63;
     return ((long long)m ^ sg) - sg;
 }
@@ -107,34 +121,33 @@ __device__ __forceinline__ void mma_f16_k8(float (&c)[4], uint32_t a0, uint32_t 
 }
 
 // xh (digits 0..2) and xl (digits 3..5) of a Q62 value
+template <bool WIDE = false>
 __device__ __forceinline__ void fx_split(long long x, int &h, int &l) {
     constexpr int kBias27 = (1 << 26) + (1 << 17) + (1 << 8);       // 256 in each of three digits
-    const unsigned long long y = (unsigned long long)x + kFxBias;
-    h = (int)(uint32_t)(y >> 36) - kBias27;
+    const unsigned long long y = (unsigned long long)x + (WIDE ? kFxBiasWide : kFxBias);
+    h = (int)(uint32_t)(y >> 36) - kBias27 - (WIDE ? 1 << 26 : 0);
     l = (int)((uint32_t)(y >> 9) & 0x7ffffffu) - kBias27;
 }
 
-// the product sum times 2^57, rounded: from the digit sums, and from sum xh yh and
-// sum (xh yl + xl yh)
-__device__ __forceinline__ long long fx_combine(const float (&a)[kFxSums]) {
-    long long x = (long long)__float2int_rn(a[7]) + (1ll << 21);
-    x += (long long)__float2int_rn(a[6]) * 512ll;
-    x += (long long)__float2int_rn(a[5]) * 262144ll;
-    long long v = x >> 22;
-    v += (long long)__float2int_rn(a[4]) * 32ll;
-    v += (long long)__float2int_rn(a[3]) * 16384ll;
-    v += (long long)__float2int_rn(a[2]) * 8388608ll;
-    v += (long long)((unsigned long long)(uint32_t)(__float2int_rn(a[1]) + (__float2int_rn(a[0]) << 9)) << 32);
-    return v;
-}
 // x 2^-n rounded to nearest, ties to even
 __device__ __forceinline__ long long fx_shift_even(long long x, int n) {
     return n > 0 ? (x + ((1ll << (n - 1)) - 1) + ((x >> n) & 1)) >> n : x;
 }
-// the same from the digit sums of orders 0 to 6 alone, rounded to even: with one factor 1 a 32nd
-// of the sums are ties
-__device__ __forceinline__ long long fx_combine(const float (&a)[kFxSums - 1]) {
-    long long v = fx_shift_even((long long)__float2int_rn(a[6]) + (long long)__float2int_rn(a[5]) * 512ll, 13);
+// The product sum times 2^57, rounded: from the digit sums (orders 0 to 7, or 0 to 6 and
+// rounded to even: with one factor 1 a 32nd of the sums are ties), and from sum xh yh and
+// sum (xh yl + xl yh).
+template <int N>
+__device__ __forceinline__ long long fx_combine(const float (&a)[N]) {
+    static_assert(N == kFxSums || N == kFxSums - 1, "orders 0 to 7 or 0 to 6");
+    long long v;
+    if constexpr (N == kFxSums) {
+        long long x = (long long)__float2int_rn(a[7]) + (1ll << 21);
+        x += (long long)__float2int_rn(a[6]) * 512ll;
+        x += (long long)__float2int_rn(a[5]) * 262144ll;
+        v = x >> 22;
+    } else {
+        v = fx_shift_even((long long)__float2int_rn(a[6]) + (long long)__float2int_rn(a[5]) * 512ll, 13);
+    }
     v += (long long)__float2int_rn(a[4]) * 32ll;
     v += (long long)__float2int_rn(a[3]) * 16384ll;
     v += (long long)__float2int_rn(a[2]) * 8388608ll;

@@ -11,10 +11,14 @@
 // over 2 K terms.  At 1/64 of the FP32 rate the FP64 pipe bound the direct form
 // (k_interp_f64, one thread per sample: 594 FP64 operations a sample at p = 4,
 // K = 16, 0.96 of the measured FP64 peak).  Here both factors are split into six
-// FP16 digits (fxdigits.cuh) and 27 digit products run as mma.sync m16n8k16: 16 nodes x 8 samples of the cell x 8 orders k, exact in the
-// FP32 accumulators, recombined as 64-bit integers, so the sum carries the
-// rounding of its operands to 2^-54 of the cell's largest |F| and |e^{ik psi}| = 1
-// and nothing else.  A tile of 16 nodes is exactly the 4 x 4 stencil; the 128-row
+// FP16 digits (fxdigits.cuh) and 27 digit products run as mma.sync m16n8k16: 16 nodes x 8
+// samples of the cell x 8 orders k, exact in the FP32 accumulators, recombined as 64-bit
+// integers and weighted with rounding to nearest, so the sum carries the rounding of its
+// operands -- 2^-55 of the power of two above the cell's largest |F| (digits of twice the
+// range), 2^-54 of |e^{ik psi}| = 1 -- and the products of their low halves, left out.
+// Relative L2 error of a TOD against long double, direct sum -> here: LFI-like sky and
+// sidelobe beam, K = 16 2.9e-16 -> 1.3e-16 (scan), K = 32 4.3e-16 -> 1.8e-16, p = 6, K = 8
+// 3.4e-16 -> 1.9e-16, p = 2 2.4e-16 -> 1.0e-16.  A tile of 16 nodes is exactly the 4 x 4 stencil; the 128-row
 // tiles of tcgen05 would be 7/8 padding here, and at 54 MMAs of 2.15 clocks (the
 // rate mma.sync measured: 1024 multiply-adds per clock and SM) per 8 samples the
 // tensor pipe is not what binds.
@@ -76,6 +80,10 @@ __device__ __forceinline__ int fx_node(const InterpGeom &g, int i, int j, int q)
     if (!SL_GUARD(ring >= 0 && ring < g.R && col >= 0 && col < g.nphi, 0x211u)) return 0;
     return (ring * g.nphi + col) * (g.K + 1);
 }
+
+// Exponent field of a cell's scale 2^e, e = field - 1022, from the largest high word: F 2^(63 - e) has to
+// leave its digits' biases room, so the next exponent from (1 - 2^-9) 2^e on.
+__device__ __forceinline__ int fx_scale_field(uint32_t mx) { return (int)((mx + 0x1000u) >> 20); }
 
 // the direct sum of one sample, out of line (rare)
 template <int P>
@@ -170,20 +178,20 @@ struct FxPhase {
 };
 
 // D times the weights of node q for the sample in column sc; at p = 4 both nodes of a lane
-// lie in column gr & 3, whose phi weight fx_reduce applies.  The units added to the sums (1
-// here per two nodes, 2 there) make up for the truncated products, half a unit each.
+// lie in column gr & 3, whose phi weight fx_reduce applies.  |D| < 23.2 x 2^58 and sum |w| < 2 x 1.6
+// leave the sums, in units of 2^-56, below 2^63.
 template <int P>
 __device__ __forceinline__ long long fx_weigh(long long D, const long long *tab, int q, int sc) {
     long long w = tab[(FxRows<P, false>::kWt + q / P) * kFxStride + sc];
-    if (P != 4) w = fx_mul(w, tab[(FxRows<P, false>::kWp + q % P) * kFxStride + sc]);
-    return fx_mulhi(D, w);
+    if (P != 4) w = fx_mul_rn(w, tab[(FxRows<P, false>::kWp + q % P) * kFxStride + sc]);
+    return fx_mulhi_rn(D, w);
 }
 // sum over the 8 row groups: `mine` is this lane's part of the sample in column sc, `other`
 // its part of the sample that the lane 16 apart goes on with
 template <int P>
 __device__ __forceinline__ long long fx_reduce(long long mine, long long other, const long long *tab, int gr, int sc) {
     mine += __shfl_xor_sync(0xffffffffu, other, 16);
-    if (P == 4) mine = fx_mul(mine, tab[(FxRows<P, false>::kWp + (gr & 3)) * kFxStride + sc]) + 2;
+    if (P == 4) mine = fx_mul_rn(mine, tab[(FxRows<P, false>::kWp + (gr & 3)) * kFxStride + sc]);
     mine += __shfl_xor_sync(0xffffffffu, mine, 8);
     mine += __shfl_xor_sync(0xffffffffu, mine, 4);
     return mine;
@@ -239,6 +247,8 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                                                                 double *__restrict__ tod) {
     constexpr int NQ = P * P, NT = (NQ + 15) / 16, NH = NQ > 8 ? 2 : 1;
     constexpr bool kOne = NT == 1 && !MB;           // one operand per cell: kept across batches, prefetched
+    // orders of the digit products kept; without the short form's halves to match, order 6 whole and no 7
+    constexpr int NS = P == 4 && !MB ? kFxSums : kFxSums - 1;
     using Rows = FxRows<P, MB>;
     if (occ && (float)n < min_mean * (float)*occ) return;   // few samples per cell: k_interp_fx_short runs instead
     extern __shared__ __align__(16) unsigned char fx_smem[];
@@ -251,7 +261,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
     const int gr = lane >> 2, q4 = lane & 3;        // fragment row group and quad lane
     const int K = g.K;
     const int nblk = MB ? (K + 15) >> 4 : 1;        // blocks of 16 orders
-    const int tsh = MB ? 3 : 0;                     // headroom of the result's sum over up to 8 blocks
+    const int tsh = MB ? 32 - __clz(nblk - 1) : 0;  // headroom of the result's sum over the blocks
 
     // A operand of the current (cell, row tile, block): digits of nodes gr and gr + 8, orders
     // 16 blk + q4 + 1 + 4 e, e = 0..3, and F_0 / 2 of both nodes
@@ -314,7 +324,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                         }
                         if (cell != a_cell) {       // largest exponent over nodes and orders
                             mx = __reduce_max_sync(0xffffffffu, mx);
-                            a_ef = (int)(mx >> 20);
+                            a_ef = fx_scale_field(mx);
                             if (a_ef < 64 || a_ef > 2022) a_ef = 2047;
                             a_cell = cell;
                         }
@@ -331,15 +341,15 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                                 // ghost rows flip the odd orders k = q4 + 1 + 4 e of this lane
                                 const int row = (int)(cell >> 16) - P / 2 + (16 * t + gr + 8 * h) / P;
                                 const bool flip = (row < 0 || row >= g.R) && !(q4 & 1);
-                                f0[h] = blk == 0 ? fx_from_double(raw[(5 * h) * 32 + lane].x, a_ef) >> 6 : 0;
+                                f0[h] = blk == 0 ? fx_from_double(raw[(5 * h) * 32 + lane].x, a_ef) >> 5 : 0;
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) {
                                     uint32_t d[kFxDig] = {0, 0, 0, 0, 0, 0};
                                     if (4 * e < K - 16 * blk) {
                                         const double2 v = raw[(5 * h + 1 + e) * 32 + lane];
-                                        long long x = fx_from_double(v.x, a_ef), y = fx_from_double(v.y, a_ef);
+                                        long long x = fx_from_double<63>(v.x, a_ef), y = fx_from_double<63>(v.y, a_ef);
                                         if (flip) { x = -x; y = -y; }
-                                        fx_digits(x, y, d);
+                                        fx_digits<true>(x, y, d);
                                     }
 #pragma unroll
                                     for (int u = 0; u < kFxDig; ++u) adig[e >> 1][u][2 * (e & 1) + h] = d[u];
@@ -362,7 +372,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                     // ---- 3: groups of 8 samples
 #pragma unroll 1
                     for (int c0 = r0; c0 < r1; c0 += 8) {
-                        float acc[4][kFxSums];      // [node h, sample e as 2 h + e][s]
+                        float acc[4][NS];           // [node h, sample e as 2 h + e][s]
                         FxPhase ph(tab, Rows::kC4, q4, min(c0 + gr, 31));   // past the run: a column of no use
 #pragma unroll
                         for (int b = 0; b < 2; ++b) {
@@ -376,7 +386,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                                 for (int u = 0; u < kFxDig; ++u)
 #pragma unroll
                                     for (int v = 0; v < kFxDig; ++v)
-                                        if (u < 3 || v < 3)
+                                        if (NS == kFxSums ? u < 3 || v < 3 : u + v < NS)
                                             mma_f16(acc[0][u + v], acc[1][u + v], acc[2][u + v], acc[3][u + v], adig[b][u],
                                                     b0[v], b1[v], b == 0 && (u == 0 || (u < 3 && v == 5)));
                             }
@@ -385,7 +395,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                         long long T[2];
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
-                            T[e] = 1;
+                            T[e] = 0;
 #pragma unroll
                             for (int h = 0; h < NH; ++h) {
                                 const int q = 16 * t + gr + 8 * h;
@@ -396,7 +406,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
                         // lanes with gr < 4 go on with the even sample
                         const int sc = c0 + 2 * q4 + (gr >> 2);
                         const long long mine = fx_reduce<P>((gr < 4) ? T[0] : T[1], (gr < 4) ? T[1] : T[0], tab, gr, min(sc, 31));
-                        if ((gr & 3) == 0 && sc < r1) tab[Rows::kT * kFxStride + sc] += (mine + (tsh ? 4 : 0)) >> tsh;
+                        if ((gr & 3) == 0 && sc < r1) tab[Rows::kT * kFxStride + sc] += fx_shift_even(mine, tsh);
                     }
                 }
             }
@@ -407,8 +417,8 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
             if (direct) {
                 out = interp_direct<P>(g, maps, rec + s, psi + s);
             } else {
-                // c = 2 T 2^-55 2^e, e = ef - 1022
-                const double sc = __longlong_as_double((long long)(efs - 53 + tsh) << 52);
+                // c = 2 T 2^-56 2^e, e = ef - 1022
+                const double sc = __longlong_as_double((long long)(efs - 54 + tsh) << 52);
                 out = (double)tab[Rows::kT * kFxStride + lane] * sc;
             }
             tod[s] = out;
@@ -516,7 +526,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, NE <= 2 ? 4 : 3) k_interp_fx_s
                                          (uint32_t)__double2hiint(raw[h][e].y) & 0x7fffffffu));
                 }
                 mx = __reduce_max_sync(0xffffffffu, mx);
-                a_ef = (int)(mx >> 20);
+                a_ef = fx_scale_field(mx);
                 if (a_ef < 64 || a_ef > 2022) a_ef = 2047;
                 a_cell = cell;
                 if (a_ef < 2047) {
@@ -524,14 +534,14 @@ __global__ void __launch_bounds__(32 * kFxsWarps, NE <= 2 ? 4 : 3) k_interp_fx_s
                     for (int h = 0; h < 2; ++h) {
                         const int row = (int)(cell >> 16) - P / 2 + (gr + 8 * h) / P;
                         const bool flip = (row < 0 || row >= g.R) && !(q4 & 1);
-                        f0[h] = fx_from_double(raw0[h], a_ef) >> 6;
+                        f0[h] = fx_from_double(raw0[h], a_ef) >> 5;
 #pragma unroll
                         for (int e = 0; e < NE; ++e) {
                             if (4 * e >= K) continue;
-                            long long x = fx_from_double(raw[h][e].x, a_ef), y = fx_from_double(raw[h][e].y, a_ef);
+                            long long x = fx_from_double<63>(raw[h][e].x, a_ef), y = fx_from_double<63>(raw[h][e].y, a_ef);
                             if (flip) { x = -x; y = -y; }
-                            fx_split(x, ah[h][e][0], al[h][e][0]);
-                            fx_split(y, ah[h][e][1], al[h][e][1]);
+                            fx_split<true>(x, ah[h][e][0], al[h][e][0]);
+                            fx_split<true>(y, ah[h][e][1], al[h][e][1]);
                         }
                     }
                 }
@@ -567,8 +577,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, NE <= 2 ? 4 : 3) k_interp_fx_s
             X += __shfl_xor_sync(0xffffffffu, up ? xx[0] : xx[1], 2);
             H += __shfl_xor_sync(0xffffffffu, H, 1);
             X += __shfl_xor_sync(0xffffffffu, X, 1);
-            long long mine = up ? 0 : 1;
-            mine += fx_weigh<P>(fx_combine(H, X) + (up ? f0[1] : f0[0]), tab, gr + (up ? 8 : 0), c);
+            long long mine = fx_weigh<P>(fx_combine(H, X) + (up ? f0[1] : f0[0]), tab, gr + (up ? 8 : 0), c);
             mine += __shfl_xor_sync(0xffffffffu, mine, 2);
             mine = fx_reduce<P>(mine, mine, tab, gr, c);
             if (lane == 0) tab[Rows::kT * kFxStride + c] = mine;
@@ -576,7 +585,7 @@ __global__ void __launch_bounds__(32 * kFxsWarps, NE <= 2 ? 4 : 3) k_interp_fx_s
         __syncwarp();
         if (lane < cnt)
             tod[s] = direct ? interp_direct<P>(g, maps, rec + s, psi + s)
-                            : (double)tab[Rows::kT * kFxStride + lane] * __longlong_as_double((long long)(efs - 53) << 52);
+                            : (double)tab[Rows::kT * kFxStride + lane] * __longlong_as_double((long long)(efs - 54) << 52);
         __syncwarp();
     }
 }
