@@ -25,6 +25,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "fxint.cuh"
+
 namespace sl {
 
 constexpr int kFxDig = 6, kFxSums = 8;
@@ -32,34 +34,6 @@ constexpr int kFxDig = 6, kFxSums = 8;
 // of X + bias unsigned 9-bit fields (10 bits for the first)
 constexpr unsigned long long kFxBias = (1ull << 62) + (1ull << 53) + (1ull << 44) + (1ull << 35) + (1ull << 26) +
                                        (1ull << 17) + (1ull << 8);
-constexpr long long kFxOne = 1ll << 62;
-
-// (a b) 2^-64 for |a|, |b| <= 2^62, at most two units off: the product of the low
-// halves is left out, and halves signed by a carry into the high ones keep all
-// three partial products signed 32 x 32 multiply-adds
-__device__ __forceinline__ long long fx_mulhi(long long a, long long b) {
-    const int al = (int)a, bl = (int)b;
-    const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31), bh = (int)(b >> 32) + (int)((unsigned)bl >> 31);
-    const long long m = (long long)ah * bl + (long long)bh * al;
-    return (long long)ah * bh + (m >> 32);
-}
-// the same rounded to nearest; |a| < 2^62.6 with |b| <= 1.5 x 2^62 is in range too
-__device__ __forceinline__ long long fx_mulhi_rn(long long a, long long b) {
-    const int al = (int)a, bl = (int)b;
-    const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31), bh = (int)(b >> 32) + (int)((unsigned)bl >> 31);
-    const long long m = (long long)ah * bl + ((long long)bh * al + (1ll << 31));
-    return (long long)ah * bh + (m >> 32);
-}
-// a b for Q62 operands (|a|, |b| <= 1): Q62, at most 2^-59 off
-__device__ __forceinline__ long long fx_mul(long long a, long long b) { return fx_mulhi(a, b) << 2; }
-// the same rounded to nearest, without the truncation's bias (zero stays zero): at most 2^-61 off
-__device__ __forceinline__ long long fx_mul_rn(long long a, long long b) {
-    const int al = (int)a, bl = (int)b;
-    const int ah = (int)(a >> 32) + (int)((unsigned)al >> 31), bh = (int)(b >> 32) + (int)((unsigned)bl >> 31);
-    const long long m = (long long)ah * bl + (long long)bh * al;
-    return (long long)ah * bh * 4 + ((m + (1ll << 29)) >> 30);
-}
-
 // Digits for operands of twice the range: x in (-2 + 2^-7, 2 - 2^-7), X = x 2^62, d_0 within
 // +-512, which FP16 and the sums above still hold (32 x (5 x 2^16 + 2^17) < 2^24).
 constexpr unsigned long long kFxBiasWide = kFxBias + (1ull << 62);
@@ -129,10 +103,6 @@ __device__ __forceinline__ void fx_split(long long x, int &h, int &l) {
     l = (int)((uint32_t)(y >> 9) & 0x7ffffffu) - kBias27;
 }
 
-// x 2^-n rounded to nearest, ties to even
-__device__ __forceinline__ long long fx_shift_even(long long x, int n) {
-    return n > 0 ? (x + ((1ll << (n - 1)) - 1) + ((x >> n) & 1)) >> n : x;
-}
 // The product sum times 2^57, rounded: from the digit sums (orders 0 to 7, or 0 to 6 and
 // rounded to even: with one factor 1 a 32nd of the sums are ties), and from sum xh yh and
 // sum (xh yl + xl yh).
@@ -151,7 +121,7 @@ __device__ __forceinline__ long long fx_combine(const float (&a)[N]) {
     v += (long long)__float2int_rn(a[4]) * 32ll;
     v += (long long)__float2int_rn(a[3]) * 16384ll;
     v += (long long)__float2int_rn(a[2]) * 8388608ll;
-    v += (long long)((unsigned long long)(uint32_t)(__float2int_rn(a[1]) + (__float2int_rn(a[0]) << 9)) << 32);
+    v += (long long)((unsigned long long)(uint32_t)(__float2int_rn(a[1]) + __float2int_rn(a[0]) * 512) << 32);
     return v;
 }
 __device__ __forceinline__ long long fx_combine(long long hh, long long x) { return hh * 32 + ((x + (1ll << 21)) >> 22); }

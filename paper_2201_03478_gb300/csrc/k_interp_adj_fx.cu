@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                         erow[(u * 8 + 2 * k) * (2 * kFaRow)] = __low2half(h);
                         erow[(u * 8 + 2 * k + 1) * (2 * kFaRow)] = __high2half(h);
                     }
-                    const long long nc = (fx_mulhi(zc, xc) << 3) - pc, ns = (fx_mulhi(zc, xs) << 3) - px;
+                    const long long nc = fx_cheb(zc, xc, pc), ns = fx_cheb(zc, xs, px);
                     pc = xc;
                     px = xs;
                     xc = nc;

@@ -121,9 +121,9 @@ __device__ __forceinline__ bool fx_setup(const InterpGeom &g, const StencilRec64
     }
     direct |= wsum >= (2ull << 60);                 // keeps the weighted sum below 2^63
     // (cos, -sin) of exponents -3 .. 4
-    const long long c2 = fx_mul(zc, zc) - fx_mul(zs, zs), s2 = fx_mul(zc, zs) << 1;
+    const long long c2 = fx_mul(zc, zc) - fx_mul(zs, zs), s2 = fx_mul(zc, zs) * 2;
     const long long c3 = fx_mul(c2, zc) - fx_mul(s2, zs), s3 = fx_mul(c2, zs) + fx_mul(s2, zc);
-    const long long c4 = fx_mul(c2, c2) - fx_mul(s2, s2), s4 = fx_mul(c2, s2) << 1;
+    const long long c4 = fx_mul(c2, c2) - fx_mul(s2, s2), s4 = fx_mul(c2, s2) * 2;
     const long long cs[4] = {kFxOne, zc, c2, c3}, ss[4] = {0, zs, s2, s3};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -139,9 +139,9 @@ __device__ __forceinline__ bool fx_setup(const InterpGeom &g, const StencilRec64
     if (MB) col[Rows::kC4 * kFxStride] = c4;
     col[Rows::kT * kFxStride] = 0;
     if (MB) {
-        const long long c8 = fx_mul(c4, c4) - fx_mul(s4, s4), s8 = fx_mul(c4, s4) << 1;
+        const long long c8 = fx_mul(c4, c4) - fx_mul(s4, s4), s8 = fx_mul(c4, s4) * 2;
         col[Rows::kZ16 * kFxStride] = fx_mul(c8, c8) - fx_mul(s8, s8);
-        col[(Rows::kZ16 + 1) * kFxStride] = fx_mul(c8, s8) << 1;
+        col[(Rows::kZ16 + 1) * kFxStride] = fx_mul(c8, s8) * 2;
     }
     return direct;
 }
@@ -169,7 +169,7 @@ struct FxPhase {
         c4 = tab[row_c4 * kFxStride + col];
     }
     __device__ __forceinline__ void step() {
-        const long long nc = (fx_mulhi(c4, c) << 3) - pc, ns = (fx_mulhi(c4, s) << 3) - ps;
+        const long long nc = fx_cheb(c4, c, pc), ns = fx_cheb(c4, s, ps);
         pc = c;
         ps = s;
         c = nc;

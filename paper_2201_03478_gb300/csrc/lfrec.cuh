@@ -33,13 +33,13 @@ __device__ __forceinline__ int4 lf_coef(double a, double b, bool &big) {
     big = a + fabs(b) >= 4.0;
     const long long A = big ? 0 : fx_from_double(a, 1026), B = big ? 0 : fx_from_double(-b, 1026);  // 2^58
     const int Ah = (int)((A + (1ll << 30)) >> 31);
-    return make_int4(Ah, (int)(A - ((long long)Ah << 31)), (int)B, (int)(B >> 32));
+    return make_int4(Ah, (int)(A - (long long)Ah * (1ll << 31)), (int)B, (int)(B >> 32));
 }
 // x in [-1, 1] as xh 2^-31 + xl 2^-62, |xl| <= 2^30
 __device__ __forceinline__ void lf_set_x(LfRec &r, double x) {
     const long long X = max(min(fx_from_double(x, 1023), (1ll << 61) - 1), 1 - (1ll << 61)) * 2;
     r.xh = (int)((X + (1ll << 30)) >> 31);
-    r.xl = (int)(X - ((long long)r.xh << 31));
+    r.xl = (int)(X - (long long)r.xh * (1ll << 31));
 }
 // y 2^(60 - U), rounded
 __device__ __forceinline__ long long lf_from_double(double y, int U) { return (fx_from_double(y, U + 1022) + 2) >> 2; }
