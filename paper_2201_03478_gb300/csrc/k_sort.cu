@@ -10,7 +10,7 @@
 //
 //   k_bin:        pointing -> (i, j) in double; key; record {theta - theta(i-1),
 //                 phi fraction, [reduced psi], cell}; key histogram
-//   k_scan_local / k_scan_add:  exclusive prefix sum of the histogram
+//   k_scan_local / (k_scan_blocks) / k_scan_add:  exclusive prefix sum of the histogram
 //                 -> first position of every key (and a cursor copy)
 //   k_scatter_agg: perm[cursor[key]++] = s, the cursor atomics aggregated per
 //                 chunk of samples in shared memory (order within a key unspecified)
@@ -191,20 +191,44 @@ __global__ void __launch_bounds__(1024) k_scan_local(int64_t n, unsigned *__rest
     }
 }
 
+// Exclusive scan of bsum[0 .. nb) in place, bsum[nb] = total, by one CTA.
+__global__ void __launch_bounds__(1024) k_scan_blocks(int nb, unsigned *__restrict__ bsum) {
+    unsigned carry = 0;
+    for (int base = 0; base < nb; base += kScanBlock) {
+        const int i = base + 4 * threadIdx.x;
+        const uint4 v = load4(bsum, i, nb);
+        unsigned ex;
+        const unsigned tot = block_exclusive_scan(v.x + v.y + v.z + v.w, ex);
+        ex += carry;
+        store4(bsum, i, nb, make_uint4(ex, ex + v.x, ex + v.x + v.y, ex + v.x + v.y + v.z));
+        carry += tot;
+    }
+    if (threadIdx.x == 0) bsum[nb] = carry;
+}
+
 // Adds the totals of the CTAs before to k_scan_local's sums and copies them to cursor; the
-// last CTA also writes data[n] = total and, with occ, *occ = the sum of nz.  Every CTA sums the
-// earlier totals itself (nb^2 / 2 words from L2, 0.5 MB at 1024 x 2048 cells): a scan of them by
-// one CTA in between, and of the tiles' chunks by another, cost the small and sparse sorts two
-// launches, and with the tiles' strided words more than the rest of the scan (1500 x 3000
-// cells: 17 + 5 + 12 + 4 + 66 us, now 10 + 11 + 37).
+// last CTA also writes data[n] = total and, with occ, *occ = the sum of nz.  Up to kScanQuadratic
+// CTAs every one sums the earlier totals itself (nb^2 / 2 words from L2, 0.5 MB at 1024 x 2048
+// cells): a scan of them by one CTA in between, and of the tiles' chunks by another, cost the small
+// and sparse sorts two launches, and with the tiles' strided words more than the rest of the scan
+// (1500 x 3000 cells: 17 + 5 + 12 + 4 + 66 us, now 10 + 11 + 37).  The work grows with the square of
+// the cells, so beyond (SCANNED) k_scan_blocks runs in between: 16384^2 cells 1.23 -> 0.95 ms,
+// 32768 x 16384 3.71 -> 1.88.
+constexpr int64_t kScanQuadratic = 65536;
+
+template <bool SCANNED>
 __global__ void __launch_bounds__(1024) k_scan_add(int64_t n, unsigned *__restrict__ data, const unsigned *__restrict__ bsum,
                                                     const unsigned *__restrict__ nz, unsigned *__restrict__ cursor,
                                                     unsigned *__restrict__ occ) {
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + 4 * threadIdx.x;
     uint4 v = load4(data, base, n);
     unsigned before = 0;
-    for (unsigned i = threadIdx.x; i < blockIdx.x; i += 1024) before += bsum[i];
-    before = block_sum(before);
+    if (SCANNED) {
+        before = bsum[blockIdx.x];
+    } else {
+        for (unsigned i = threadIdx.x; i < blockIdx.x; i += 1024) before += bsum[i];
+        before = block_sum(before);
+    }
     v = make_uint4(before + v.x, before + v.y, before + v.z, before + v.w);
     store4(data, base, n, v);
     store4(cursor, base, n, v);
@@ -215,7 +239,7 @@ __global__ void __launch_bounds__(1024) k_scan_add(int64_t n, unsigned *__restri
         o = block_sum(o);
         if (threadIdx.x == 0) *occ = o;
     }
-    if (threadIdx.x == 0) data[n] = before + bsum[blockIdx.x];
+    if (threadIdx.x == 0) data[n] = SCANNED ? bsum[gridDim.x] : before + bsum[blockIdx.x];
 }
 
 // The scatter with its atomics aggregated per chunk of kAggChunk samples: a
@@ -302,22 +326,41 @@ __global__ void __launch_bounds__(kAggThreads) k_scatter_agg(int64_t n, int64_t 
 }
 
 // chunk_off[t] = sum over the tiles before t of ceil(#samples / kChunk), chunk_off[ntiles] = total.
-// One CTA per 1024 tiles, which also sums the chunks of the tiles before its own (37 us at 1500 x
-// 3000 cells, bound by its strided reads; the counts and a single CTA's scan took 4 + 66).
+// One CTA per 1024 tiles, which up to kTilesQuadratic tiles also sums the chunks of the tiles before its
+// own (37 us at 1500 x 3000 cells, bound by its strided reads; the counts and a single CTA's scan
+// took 4 + 66).  That is the square of the tiles (3000 x 6000 cells still as fast, 4096 x 8192 0.06 ms
+// slower, 32768 x 16384 63 ms of a call of 73), so beyond (tot given) the CTAs scan their own tiles and
+// leave their totals, and k_chunk_add adds those before (calls of 1e5 FP32 samples: 4096 x 8192 cells
+// 1.63 -> 1.24 ms, 8192 x 16384 5.9 -> 2.0, 32768 x 16384 73 -> 4.0).
+constexpr int kTilesQuadratic = 160000;
+
 __global__ void __launch_bounds__(1024) k_tile_chunks(int ntiles, int ncell, const unsigned *__restrict__ start,
-                                                       unsigned *__restrict__ chunk_off) {
+                                                       unsigned *__restrict__ chunk_off, unsigned *__restrict__ tot) {
     auto chunks = [&](int t) {
         return (start[(int64_t)(t + 1) * ncell] - start[(int64_t)t * ncell] + kChunk - 1) / kChunk;
     };
     const int t0 = blockIdx.x * 1024, t = t0 + threadIdx.x;
     unsigned before = 0;
+    if (!tot) {
 #pragma unroll 4
-    for (int i = threadIdx.x; i < t0; i += 1024) before += chunks(i);
-    before = block_sum(before);
+        for (int i = threadIdx.x; i < t0; i += 1024) before += chunks(i);
+        before = block_sum(before);
+    }
     unsigned ex;
-    const unsigned tot = block_exclusive_scan(t < ntiles ? chunks(t) : 0u, ex);
+    const unsigned own = block_exclusive_scan(t < ntiles ? chunks(t) : 0u, ex);
     if (t < ntiles) chunk_off[t] = before + ex;
-    if (threadIdx.x == 0 && t0 + 1024 >= ntiles) chunk_off[ntiles] = before + tot;
+    if (threadIdx.x != 0) return;
+    if (tot) tot[blockIdx.x] = own;
+    else if (t0 + 1024 >= ntiles) chunk_off[ntiles] = before + own;
+}
+
+__global__ void __launch_bounds__(1024) k_chunk_add(int ntiles, const unsigned *__restrict__ tot, unsigned *__restrict__ chunk_off) {
+    unsigned before = 0;
+    for (unsigned i = threadIdx.x; i < blockIdx.x; i += 1024) before += tot[i];
+    before = block_sum(before);
+    const int t = blockIdx.x * 1024 + threadIdx.x;
+    if (t < ntiles) chunk_off[t] += before;
+    if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) chunk_off[ntiles] = before + tot[blockIdx.x];
 }
 
 SL_CHECK_READER(chk_sort)
@@ -352,7 +395,12 @@ sl_status launch_sort_into(sl_plan *p, const SortBufs &b, const double *theta, c
     slot = timing_begin(p, "scan");
     unsigned *nz = b.occ ? b.occ + 1 : nullptr;
     k_scan_local<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, nz);
-    k_scan_add<<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, nz, b.cursor, b.occ);
+    if (nb > kScanQuadratic) {
+        k_scan_blocks<<<1, 1024, 0, p->stream>>>((int)nb, b.bsum);
+        k_scan_add<true><<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, nz, b.cursor, b.occ);
+    } else {
+        k_scan_add<false><<<(unsigned)nb, 1024, 0, p->stream>>>(nkeys, b.hist, b.bsum, nz, b.cursor, b.occ);
+    }
     timing_end(p, slot);
     if ((st = cuda_check(cudaGetLastError(), "k_scan launch")) != SL_OK) return st;
     slot = timing_begin(p, "scatter");
@@ -369,7 +417,11 @@ sl_status launch_sort_into(sl_plan *p, const SortBufs &b, const double *theta, c
     timing_end(p, slot);
     if ((st = cuda_check(cudaGetLastError(), "k_scatter_agg launch")) != SL_OK) return st;
     if (with_chunks) {
-        k_tile_chunks<<<(p->ntiles + 1023) / 1024, 1024, 0, p->stream>>>(p->ntiles, ncell, b.hist, b.chunk_off);
+        // the totals go over the block sums, which are done with: 1024 tiles take more than 4096 keys
+        const unsigned nc = (unsigned)((p->ntiles + 1023) / 1024);
+        const bool apart = fine && p->ntiles > kTilesQuadratic;
+        k_tile_chunks<<<nc, 1024, 0, p->stream>>>(p->ntiles, ncell, b.hist, b.chunk_off, apart ? b.bsum : nullptr);
+        if (apart) k_chunk_add<<<nc, 1024, 0, p->stream>>>(p->ntiles, b.bsum, b.chunk_off);
         st = cuda_check(cudaGetLastError(), "k_tile_chunks launch");
     }
     return st;
