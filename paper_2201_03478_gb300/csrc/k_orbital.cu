@@ -142,16 +142,16 @@ __global__ void __launch_bounds__(256) k_orb_nodes(const OrbArgs a) {
     }
 }
 
-constexpr int kOrbThreads = 256;
-constexpr int kOrbRound = kOrbThreads * kOrbRun;  // rows per sweep round
-
 // shared-memory slot of round row q: one pad slot per thread's run, so that the lanes'
 // rows (8 l + i) fall on distinct banks
 __device__ __forceinline__ int orb_pad(int q) { return q + (q >> 3); }
-constexpr int kOrbPad = kOrbRound + kOrbRound / kOrbRun + 2;
+// threads per period: one warp up to kOrbShortNodes nodes (one round of it), eight beyond.  A short
+// period leaves most of eight warps at barriers: 1e7 samples in periods of 100 (5 nodes, s = 20) 1181 -> 348
+// us, of 1950 (98 nodes) 97 -> 51, of 4000 (200 nodes) 58 -> 30.
+constexpr int kOrbThreads = 256, kOrbShortThreads = 32;
 
 // The value that enters this thread's rows, from every thread's (end value from zero A, factor F)
-// and the value that enters the round; ends[warp]: the warps' end values (ends[7]: the round's).
+// and the value that enters the round; ends[warp]: the warps' end values (the last one the round's).
 __device__ __forceinline__ double orb_enter(double A, double F, double carry, double *ends) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -169,19 +169,21 @@ __device__ __forceinline__ double orb_enter(double A, double F, double carry, do
     return lane ? fma(pf, in, pa) : in;
 }
 
-// One CTA per period: both sweeps in rounds of kOrbRound rows, values staged through shared
+// One CTA of NT threads per period: both sweeps in rounds of NT x kOrbRun rows, values staged through shared
 // memory so that global accesses are coalesced.  The forward sweep's dp_j wait in the first
 // quarter of the period's cubics: cubic j (doubles 4 j .. 4 j + 3) replaces dp values of rows at
 // or above j, which the backward sweep has read by then.
-__global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
+template <int NT>
+__global__ void __launch_bounds__(NT) k_orb_spline(const OrbArgs a) {
+    constexpr int ROUND = NT * kOrbRun, PAD = ROUND + ROUND / kOrbRun + 2;
     __shared__ double s_piv[kOrbPivots];
-    __shared__ double s_y[kOrbPad], s_d[kOrbPad];
-    __shared__ double s_end[2][kOrbThreads / 32];
-    for (int j = threadIdx.x; j < kOrbPivots; j += kOrbThreads) s_piv[j] = a.piv[j];
-    __syncthreads();
+    __shared__ double s_y[PAD], s_d[PAD];
+    __shared__ double s_end[2][NT / 32];
     const int64_t p = blockIdx.x;
     const int64_t g0 = a.noff[p], M = a.noff[p + 1] - g0;
-    if (M < 2) return;
+    if (M < 2 || (M <= kOrbShortNodes) != (NT == kOrbShortThreads)) return;     // nothing to do, or the other launch's
+    for (int j = threadIdx.x; j < kOrbPivots; j += NT) s_piv[j] = a.piv[j];
+    __syncthreads();
     const double *__restrict__ y = a.y + g0;
     double4_32a *cub = a.cub + g0;
     double *dp = reinterpret_cast<double *>(cub);
@@ -190,9 +192,9 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
     int par = 0;                                     // s_end is used alternately: one barrier a round less
     // forward sweep over rows 1 .. M-2: dp_j = (rhs_j - dp_{j-1}) c_j, dp_0 = 0
     double carry = 0.0;
-    for (int64_t base = 1; base <= M - 2; base += kOrbRound, par ^= 1) {
-        const int rows = (int)min((int64_t)kOrbRound, M - 1 - base);
-        for (int k = threadIdx.x; k < rows + 2; k += kOrbThreads) s_y[orb_pad(k)] = y[base - 1 + k];
+    for (int64_t base = 1; base <= M - 2; base += ROUND, par ^= 1) {
+        const int rows = (int)min((int64_t)ROUND, M - 1 - base);
+        for (int k = threadIdx.x; k < rows + 2; k += NT) s_y[orb_pad(k)] = y[base - 1 + k];
         __syncthreads();
         double v[kOrbRun], d = 0.0, f = 1.0;
 #pragma unroll
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
                 v[i] = d;
             }
         double in = orb_enter(d, f, carry, s_end[par]);
-        carry = s_end[par][kOrbThreads / 32 - 1];
+        carry = s_end[par][NT / 32 - 1];
 #pragma unroll
         for (int i = 0; i < kOrbRun; ++i)
             if (lo + i < rows) {
@@ -213,17 +215,17 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
                 s_d[orb_pad(lo + i)] = v[i] + in;
             }
         __syncthreads();
-        for (int k = threadIdx.x; k < rows; k += kOrbThreads) dp[base + k] = s_d[orb_pad(k)];
+        for (int k = threadIdx.x; k < rows; k += NT) dp[base + k] = s_d[orb_pad(k)];
     }
     __syncthreads();                                 // dp is read by other threads than wrote it
     // backward sweep: N_j = dp_j - c_j N_{j+1}, N_{M-1} = 0; round row q is j = top - q, then the
     // cubics of nodes top .. top - rows + 1, from N_j and N_{j+1}
     carry = 0.0;
     double above = 0.0;                              // N of the row above the round
-    for (int64_t top = M - 2; top >= 1; top -= kOrbRound, par ^= 1) {
-        const int rows = (int)min((int64_t)kOrbRound, top);
-        for (int k = threadIdx.x; k < rows; k += kOrbThreads) s_d[orb_pad(k)] = dp[top - k];
-        for (int k = threadIdx.x; k < rows + 1; k += kOrbThreads) s_y[orb_pad(k)] = y[top + 1 - k];
+    for (int64_t top = M - 2; top >= 1; top -= ROUND, par ^= 1) {
+        const int rows = (int)min((int64_t)ROUND, top);
+        for (int k = threadIdx.x; k < rows; k += NT) s_d[orb_pad(k)] = dp[top - k];
+        for (int k = threadIdx.x; k < rows + 1; k += NT) s_y[orb_pad(k)] = y[top + 1 - k];
         __syncthreads();
         double v[kOrbRun], m = 0.0, f = 1.0;
 #pragma unroll
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
                 v[i] = m;
             }
         double in = orb_enter(m, f, carry, s_end[par]);
-        carry = s_end[par][kOrbThreads / 32 - 1];
+        carry = s_end[par][NT / 32 - 1];
 #pragma unroll
         for (int i = 0; i < kOrbRun; ++i)
             if (lo + i < rows) {
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_spline(const OrbArgs a) {
                 s_d[orb_pad(lo + i)] = v[i] + in;
             }
         __syncthreads();
-        for (int k = threadIdx.x; k < rows; k += kOrbThreads) {
+        for (int k = threadIdx.x; k < rows; k += NT) {
             const double m0 = s_d[orb_pad(k)], m1 = k ? s_d[orb_pad(k - 1)] : above;
             const double y0 = s_y[orb_pad(k + 1)], y1 = s_y[orb_pad(k)];
             cub[top - k] = make_double4_32a(y0, (y1 - y0) - fma(2.0, m0, m1), 3.0 * m0, m1 - m0);
@@ -336,7 +338,8 @@ sl_status launch_orbital(sl_plan *p, const OrbLaunch &o) {
         sl_status st = cuda_check(cudaGetLastError(), "k_orb_nodes launch");
         if (st != SL_OK) return st;
         slot = timing_begin(p, "orb_spline");
-        k_orb_spline<<<(unsigned)a.nper, kOrbThreads, 0, p->stream>>>(a);
+        if (o.nshort > 0) k_orb_spline<kOrbShortThreads><<<(unsigned)a.nper, kOrbShortThreads, 0, p->stream>>>(a);
+        if (o.nlong > 0) k_orb_spline<kOrbThreads><<<(unsigned)a.nper, kOrbThreads, 0, p->stream>>>(a);
         timing_end(p, slot);
         if ((st = cuda_check(cudaGetLastError(), "k_orb_spline launch")) != SL_OK) return st;
     }
