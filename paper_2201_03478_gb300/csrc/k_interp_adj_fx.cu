@@ -38,7 +38,7 @@
 namespace sl {
 
 constexpr int kFaWarps = 4;
-constexpr int kFaRow = 20;         // words per row of 32 samples (padded: fragment rows in distinct banks)
+constexpr int kFaRow = 16;         // words per row of 32 samples, swizzled (fa_word)
 constexpr int kFaDig = 7;          // digits of y w (the phases have six); products of orders 0 to 6
 constexpr int kFaEmpty = -4096;    // exponent of sums that are all zero
 constexpr int kFaChunk = 512;      // longest stretch of a warp: keeps the 64-bit sums in range
@@ -47,6 +47,9 @@ struct FaWarp {                    // one warp's shared memory; sums follow (fa_
     uint32_t a[kFaDig][16][kFaRow];     // digits of y w: [digit][4 row + column mod 4][sample pair]
     uint32_t e[6][8][kFaRow];      // digits of the phases of 4 orders: [digit][2 order + part][sample pair]
 };
+// Word w of row r: the eight rows and four words of a fragment in distinct banks, without padding
+// (rows of 20 words took a fifth more shared memory, and the fourth CTA of an SM up to 8 orders).
+__device__ __forceinline__ int fa_word(int r, int w) { return w ^ (((r >> 1) & 3) << 2); }
 // bytes per warp with the sums of order 0 (2 rows) and of blocks of 4 orders (2 rows x re, im)
 __host__ __device__ __forceinline__ size_t fa_warp_bytes(int nblk) {
     return sizeof(FaWarp) + (size_t)(2 + 4 * nblk) * 32 * sizeof(long long);
@@ -203,7 +206,14 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
             // its 62 bits enter the seven digits (1e7 uniform samples on 127 x 128 cells, cube against long
             // double: 5.9e-16; six digits, 2^-53 of twice the run's largest |y|: 16e-16; FP64: 6.7e-16).
             const long long yq = use ? fx_from_double(y, ey) >> 1 : 0;
-            __half *arow = reinterpret_cast<__half *>(&W.a[0][0][lane >> 1]) + (lane & 1);
+            // halves of row 4 a + slot from row 4 a on: an odd a flips the third bit of the word (fa_word)
+            __half *arow = reinterpret_cast<__half *>(W.a) + (lane & 1);
+            int off[4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int slot = (j - 1 + b) & 3;
+                off[b] = 2 * (slot * kFaRow + fa_word(slot, lane >> 1));
+            }
 #pragma unroll 1
             for (int a = 0; a < 4; ++a) {
                 const long long ya = fx_mul_rn(yq, lwt[0]);
@@ -214,8 +224,7 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                 for (int b = 0; b < 4; b += 2) {
                     uint32_t d[kFaDig];
                     fx_digits(fx_mul_rn(ya, lwp[b]), fx_mul_rn(ya, lwp[b + 1]), d);
-                    __half *o0 = arow + (4 * a + ((j - 1 + b) & 3)) * (2 * kFaRow);
-                    __half *o1 = arow + (4 * a + ((j + b) & 3)) * (2 * kFaRow);
+                    __half *o0 = arow + (off[b] ^ ((a & 1) << 4)), *o1 = arow + (off[b + 1] ^ ((a & 1) << 4));
 #pragma unroll
                     for (int u = 0; u < kFaDig; ++u) {
                         const __half2 h = *reinterpret_cast<const __half2 *>(&d[u]);
@@ -223,6 +232,7 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                         o1[u * (16 * 2 * kFaRow)] = __high2half(h);
                     }
                 }
+                arow += 4 * 2 * kFaRow;
             }
         }
         if (t0 + 32 < wlast) {
@@ -231,7 +241,7 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
             ps_next = A.psi[s_next];
             y_next = A.y[s_next];
         }
-        __half *erow = reinterpret_cast<__half *>(&W.e[0][0][lane >> 1]) + (lane & 1);
+        __half *erow = reinterpret_cast<__half *>(W.e) + (lane & 1);
         long long xc = zc, xs = -zs, pc = kFxOne, px = 0;
         // ---- 2: order 0 (E = 1: the first digit 256 alone, FP16 0x5c00, in column 0), then blocks of
         // four orders
@@ -247,8 +257,9 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
 #pragma unroll
                     for (int u = 0; u < kFxDig; ++u) {
                         const __half2 h = *reinterpret_cast<const __half2 *>(&d[u]);
-                        erow[(u * 8 + 2 * k) * (2 * kFaRow)] = __low2half(h);
-                        erow[(u * 8 + 2 * k + 1) * (2 * kFaRow)] = __high2half(h);
+                        __half *o = erow + 2 * ((u * 8 + 2 * k) * kFaRow + fa_word(2 * k, lane >> 1));   // 2 k + 1: the same swizzle
+                        o[0] = __low2half(h);
+                        o[2 * kFaRow] = __high2half(h);
                     }
                     const long long nc = fx_cheb(zc, xc, pc), ns = fx_cheb(zc, xs, px);
                     pc = xc;
@@ -301,13 +312,14 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                     const int p0 = 16 * t + 2 * q4, p1 = p0 + 8;
                     const uint32_t m0 = (p0 >= r0 && p0 < r1 ? 0xffffu : 0u) | (p0 + 1 >= r0 && p0 + 1 < r1 ? 0xffff0000u : 0u);
                     const uint32_t m1 = (p1 >= r0 && p1 < r1 ? 0xffffu : 0u) | (p1 + 1 >= r0 && p1 + 1 < r1 ? 0xffff0000u : 0u);
+                    const int w0 = fa_word(gr, 8 * t + q4);     // rows gr and gr + 8: the same swizzle
                     uint32_t ad[kFaDig][4];
 #pragma unroll
                     for (int u = 0; u < kFaDig; ++u) {
-                        ad[u][0] = W.a[u][gr][8 * t + q4] & m0;
-                        ad[u][1] = W.a[u][gr + 8][8 * t + q4] & m0;
-                        ad[u][2] = W.a[u][gr][8 * t + q4 + 4] & m1;
-                        ad[u][3] = W.a[u][gr + 8][8 * t + q4 + 4] & m1;
+                        ad[u][0] = W.a[u][gr][w0] & m0;
+                        ad[u][1] = W.a[u][gr + 8][w0] & m0;
+                        ad[u][2] = W.a[u][gr][w0 ^ 4] & m1;
+                        ad[u][3] = W.a[u][gr + 8][w0 ^ 4] & m1;
                     }
                     if (b < 0) {
                         const uint32_t one = gr == 0 ? 0x5c005c00u : 0u;
@@ -317,7 +329,7 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
                     } else {
 #pragma unroll
                         for (int w = 0; w < kFxDig; ++w) {
-                            const uint32_t b0 = W.e[w][gr][8 * t + q4], b1 = W.e[w][gr][8 * t + q4 + 4];
+                            const uint32_t b0 = W.e[w][gr][w0], b1 = W.e[w][gr][w0 ^ 4];
 #pragma unroll
                             for (int u = 0; u < kFaDig; ++u)
                                 if (u + w < kFaDig)
