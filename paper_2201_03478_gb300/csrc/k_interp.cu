@@ -31,7 +31,7 @@ constexpr int kChunkA = kWorkChunk;
 
 // ------------------------------------------------------------------ forward FP64
 // One thread per sample: for a sort by tile (interp_tod_noalloc), where the samples of a
-// cell are not adjacent, and where interp_uses_fx finds the cell products no faster.
+// cell are not adjacent, and where interp_route finds the cell products no faster.
 template <int P>
 __global__ void __launch_bounds__(256) k_interp_f64(const InterpGeom g, const double2 *__restrict__ maps,
                                                     const StencilRec64 *__restrict__ rec,
@@ -890,13 +890,20 @@ static sl_status launch_interp_f64(sl_plan *p, const SortBufs &b, const void *ma
 }
 
 int interp_needs_chunks(const sl_plan *p, int64_t n_total) {
-    return plan_fp32(p->precision) || (p->precision == SL_DF64 && !interp_uses_fx(p, n_total));
+    float min_mean;
+    return plan_fp32(p->precision) || (p->precision == SL_DF64 && interp_route(p, n_total, &min_mean) != InterpRoute::fx);
 }
 
 sl_status launch_interp(sl_plan *p, const SortBufs &b, int fine, const void *maps, const double *psi, int64_t n,
                         int64_t n_total, double *tod) {
-    if (fine && interp_uses_fx(p, n_total)) return launch_interp_fx(p, b, maps, psi, n, tod);
-    if (p->precision == SL_DF64) return launch_interp_df(p, b, fine, maps, psi, n, tod);
+    float min_mean = 0.f;
+    const InterpRoute route = fine ? interp_route(p, n_total, &min_mean) : InterpRoute::plain;
+    const unsigned *occ = route == InterpRoute::by_occupancy ? b.occ : nullptr;
+    if (route != InterpRoute::plain) {
+        const sl_status st = launch_interp_fx(p, b, maps, psi, n, occ, min_mean, tod);
+        if (st != SL_OK || route == InterpRoute::fx) return st;
+    }
+    if (p->precision == SL_DF64) return launch_interp_df(p, b, fine, maps, psi, n, occ, min_mean, tod);
     if (p->precision == SL_FP64) {
         return launch_interp_f64(p, b, maps, psi, n, tod);
     } else {

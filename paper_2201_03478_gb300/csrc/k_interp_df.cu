@@ -26,7 +26,7 @@ struct DfArgs {
     int ntiles, ncell;
     double *tod;       // forward: written; adjoint: the input TOD
     double2 *fbar;     // adjoint cube (adjoint only)
-    const unsigned *occ;   // adjoint, with min_mean: k_interp_adj_fx runs instead if n >= min_mean *occ
+    const unsigned *occ;   // with min_mean: the fixed-point kernel runs instead if n >= min_mean *occ
     float min_mean;
     int64_t n;
 };
@@ -70,6 +70,7 @@ template <int TC, int P>
 __global__ void __launch_bounds__(256) k_interp_df_tiled(const DfArgs A) {
     constexpr int TW = TC + P - 1, NR = kTileRows + P - 1, NN = NR * TW;
     const InterpGeom &g = A.g;
+    if (A.occ && (float)A.n >= A.min_mean * (float)*A.occ) return;
     const int K1 = g.K + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *node = reinterpret_cast<float4 *>(smem_raw);   // [K1][NR][TW]
@@ -371,7 +372,7 @@ size_t interp_df_tiled_smem_tc(const sl_plan *p, int tc) {
 }
 
 sl_status launch_interp_df(sl_plan *p, const SortBufs &b, int fine, const void *maps, const double *psi, int64_t n,
-                           double *tod) {
+                           const unsigned *occ, float min_mean, double *tod) {
     if (!b.chunk_off) return set_error(SL_ERR_ARG, "double-float interpolation needs the per-tile work list");
     DfArgs a;
     a.g = p->geom;
@@ -385,6 +386,9 @@ sl_status launch_interp_df(sl_plan *p, const SortBufs &b, int fine, const void *
     a.ncell = fine ? kTileRows * p->geom.tile_cols : 1;
     a.tod = tod;
     a.fbar = nullptr;
+    a.occ = occ;
+    a.min_mean = min_mean;
+    a.n = n;
     const size_t sm = interp_df_tiled_smem_tc(p, p->geom.tile_cols);
     void (*kern)(const DfArgs) = nullptr;
 #define SL_TILED(TCV, PV) \
@@ -403,7 +407,6 @@ sl_status launch_interp_df(sl_plan *p, const SortBufs &b, int fine, const void *
     const int slot = timing_begin(p, "interp_df");
     kern<<<(unsigned)(nsm * per_sm), 256, sm, p->stream>>>(a);
     timing_end(p, slot);
-    (void)n;
     return cuda_check(cudaGetLastError(), "k_interp_df launch");
 }
 

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2) k_interp_fx(const __grid_con
     // orders of the digit products kept; without the short form's halves to match, order 6 whole and no 7
     constexpr int NS = P == 4 && !MB ? kFxSums : kFxSums - 1;
     using Rows = FxRows<P, MB>;
-    if (occ && (float)n < min_mean * (float)*occ) return;   // few samples per cell: k_interp_fx_short runs instead
+    if (occ && (float)n < min_mean * (float)*occ) return;   // few samples per cell: another kernel runs instead
     extern __shared__ __align__(16) unsigned char fx_smem[];
     longlong2 *ptab = reinterpret_cast<longlong2 *>(fx_smem);       // (cos, sin)(2 pi i / 256), Q62
     for (int q = threadIdx.x; q < 256; q += 32 * kFxWarps) ptab[q] = __ldg(g.phase_tab + q);
@@ -625,34 +625,52 @@ constexpr int64_t kFxFew = 20480;   // some 8 samples a warp of k_interp_fx
 
 // Which calls take the fixed-point sums (FP64 plans otherwise k_interp_f64, DF64 plans
 // k_interp_df).  A cell's operand costs the same at every K, so few orders need many samples per
-// cell.  At p = 4 the line is the density of uniform samples (the slowest form: a scan fills
-// fewer cells) at which they break even (time over the direct sum's, FP64, 127 x 128, 256 x
+// cell.  At p = 4 and below 11 orders the line is the density of uniform samples (the slowest form: a
+// scan fills fewer cells) at which they break even (time over the direct sum's, FP64, 127 x 128, 256 x
 // 512 and 1024 x 2048 cells): K = 1 1.19, 0.86 at 61 and 122 per cell; K = 2 1.19, 0.94 at 37 and
 // 61; K = 3 1.26, 0.89 at 6 and 12; K = 4 1.02, 0.84 at 2.3 and 4.6; K = 8 1.14, 0.89 at 0.5 and
-// 1.4; K = 12 1.10, 0.80 at 0.14 and 1.4; K = 16 1.09, 0.76 (a 55-minute scan period: 0.39).
-// K = 0 gains nothing.  With at most some 8 samples for every warp of the chip, the products of
-// a cell take less time than one thread's sums: from 4 orders on 12 against 21 us (1000 samples; uniform
-// ones even out at 7e3 with K = 4 and at 1.4e4 with K = 8; a scan still gains a fifth at 2e4).
+// 1.4.  K = 0 gains nothing.  With at most some 8 samples for every warp of the chip (kFxFew), the
+// products of a cell take less time than one thread's sums: from 4 orders on 12 against 21 us (1000
+// samples); a scan gains to the end of that range, uniform samples even out at 1e4 with K = 4 and 5, 1.4e4
+// with 6 and 2e4 with 8 and lose up to 6 us of a call beyond, which stays so that these calls give a
+// sample one value whatever their size.
+// From 11 orders on the fixed-point sums are always taken.  Sparse uniform samples, nearly every one in
+// a cell of its own, lose by it (interp_tod's time over that with the direct sum at 1.12, 1.33 and 1.71 samples
+// per occupied cell, 300 x 600 cells: K = 11 1.15, 1.14, 0.97; 12 1.05, 1.10, 0.91; 14 1.09, 1.14, 0.94; 16 1.04, 1.04,
+// 0.86; 1024 x 2048: 1.15, 1.07, 0.94; 1.08, 1.00, 0.89; 1.14, 1.06, 0.93; 1.04, 0.96, 0.84), a scan at the same size gains
+// up to half (one pointing period, 0.05 per grid cell: 0.53).  Only the sort's count of occupied cells
+// tells them apart: a launch of the direct sum beside the others costs every such call 4 us (5% of a
+// scan's), and inside k_interp_fx, whose shared memory takes its L1, it is 2 to 3 times slower.
 // For p = 2 and 6 and beyond 16 orders there is only the tensor-core
 // form, whose operands cost several row tiles or blocks per cell: from 48 samples per grid
 // cell on (K = 32, p = 6, 55 per cell: 22 [43] ms; 5.5 per cell: 11 [4.4]; K = 8, p = 2: 1.6 [2.3]
-// and 0.60 [0.24]), 96 below 8 orders (K = 4: 1.26 at 61, 0.91 at 122), none below 3 (K = 2: 1.2 at 122).  DF64's alternative is faster: 13 to 16 orders from 8 samples per cell on
-// (1e8 scan samples 18.2 [32.0]; 2e7: 3.6 [6.4]; uniform ones break even at 60 per cell, 1.18 at
-// 23), 8 orders lose 1.35 at 61 per cell.  Grid cells, not occupied ones, and the whole TOD's
-// samples, so that the choice is known to the host and every piece of a TOD gets the same
-// kernel.
-bool interp_uses_fx(const sl_plan *p, int64_t n_total) {
-    if (plan_fp32(p->precision)) return false;
-    const double per_cell = (double)n_total / ((double)(p->R + 1) * p->nphi);
-    if (p->precision == SL_DF64) return p->p == 4 && p->K > 12 && p->K <= 16 && per_cell >= 8.0;
-    if (p->p != 4 || p->K > 16) return p->K > 2 && per_cell >= (p->K < 8 ? 96.0 : 48.0);
-    if (p->K == 0) return false;
-    if (p->K >= 4 && n_total <= kFxFew) return true;
+// and 0.60 [0.24]), 96 below 8 orders (K = 4: 1.26 at 61, 0.91 at 122), none below 3 (K = 2: 1.2 at 122).
+// DF64's alternative is faster: 13 to 16 orders from 8 samples per grid cell on, and there by the
+// occupied cells again, with both forms launched (time of k_interp_fx over the double-float form's, uniform samples
+// at 16, 30 and 60 per cell, 300 x 600 cells: K = 13 1.35, 1.22, 0.95; K = 16 1.17, 1.03, 0.79; 1024 x 2048, beyond L2: 0.95,
+// 0.94, 0.82; 0.79, 0.80, 0.70, and at 8 1.4 and 1.25; a scan, 200 and more per occupied cell: 0.36-0.70); 8
+// orders lose 1.35 at 61 per cell.
+// What the host decides, it decides by the whole TOD's samples per grid cell, so that every piece of a
+// TOD gets the same kernels.
+InterpRoute interp_route(const sl_plan *p, int64_t n_total, float *min_mean) {
+    *min_mean = 0.f;
+    if (plan_fp32(p->precision)) return InterpRoute::plain;
+    const double cells = (double)(p->R + 1) * p->nphi, per_cell = (double)n_total / cells;
+    if (p->precision == SL_DF64) {
+        if (p->p != 4 || p->K <= 12 || p->K > 16 || per_cell < 8.0) return InterpRoute::plain;
+        const bool in_l2 = 16.0 * (double)p->R * p->nphi * (p->K + 1) <= 1e8;       // the cube
+        *min_mean = in_l2 ? 56.f - 8.f * (float)(p->K - 13) : 16.f;
+        return per_cell >= (double)*min_mean ? InterpRoute::fx : InterpRoute::by_occupancy;     // occupied <= all cells
+    }
+    if (p->p != 4 || p->K > 16)
+        return p->K > 2 && per_cell >= (p->K < 8 ? 96.0 : 48.0) ? InterpRoute::fx : InterpRoute::plain;
+    if (p->K >= 4 && n_total <= kFxFew) return InterpRoute::fx;
     constexpr double kLine[11] = {0.0, 96.0, 48.0, 8.0, 4.0, 4.0, 4.0, 4.0, 2.0, 2.0, 2.0};
-    return p->K > 10 || per_cell >= kLine[p->K];
+    return p->K > 10 || (p->K > 0 && per_cell >= kLine[p->K]) ? InterpRoute::fx : InterpRoute::plain;
 }
 
-sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n, double *tod) {
+sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n, const unsigned *occ,
+                           float min_mean, double *tod) {
     void (*kern)(const InterpGeom, const double2 *, const StencilRec64 *, const double *, const unsigned *, int64_t, int,
                  const unsigned *, float, double *) = nullptr;
     const bool mb = p->K > 16;
@@ -682,7 +700,7 @@ sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, cons
     // the SMs both are launched, and the sort's count of occupied cells decides on the device
     // which one runs (the other returns at once).
     constexpr float kMean = 24.f;
-    const bool both = p->p == 4 && !mb && n > 4 * full && (float)n < kMean * (float)p->nkeys;
+    const bool both = p->p == 4 && !mb && p->precision != SL_DF64 && n > 4 * full && (float)n < kMean * (float)p->nkeys;
     if (both) {
         const int ne = std::max(1, (p->K + 3) / 4), ctas = nsm * (ne <= 2 ? 4 : 3);
         auto short_kern = ne == 1 ? k_interp_fx_short<1> : ne == 2 ? k_interp_fx_short<2> : ne == 3 ? k_interp_fx_short<3>
@@ -702,7 +720,7 @@ sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, cons
     const unsigned grid = (unsigned)((nwarps + kFxWarps - 1) / kFxWarps);
     int slot = timing_begin(p, "interp_fx");
     kern<<<grid, 32 * kFxWarps, sm, p->stream>>>(p->geom, (const double2 *)maps, (const StencilRec64 *)b.rec, psi, b.perm, n,
-                                                 chunk, both ? b.occ : nullptr, kMean, tod);
+                                                 chunk, both ? b.occ : occ, both ? kMean : min_mean, tod);
     timing_end(p, slot);
     return cuda_check(cudaGetLastError(), "k_interp_fx launch");
 }

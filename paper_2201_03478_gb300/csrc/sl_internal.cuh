@@ -458,10 +458,13 @@ sl_status launch_interp(sl_plan *p, const SortBufs &b, int fine, const void *map
                         int64_t n_total, double *tod);
 // whether that interpolation of a sort by cell reads the sort's work items (chunk_off)
 int interp_needs_chunks(const sl_plan *p, int64_t n_total);
-// FP64 and DF64 plans over a sort by cell: the sums on the tensor cores (k_interp_fx.cu),
-// where interp_uses_fx
-bool interp_uses_fx(const sl_plan *p, int64_t n_total);
-sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n, double *tod);
+// FP64 and DF64 plans over a sort by cell: the direct (double-float) sums, the fixed-point ones
+// (k_interp_fx.cu), or (DF64) both launched and the sort's occupied cells deciding: fixed point if n >=
+// min_mean *occ.
+enum class InterpRoute { plain, fx, by_occupancy };
+InterpRoute interp_route(const sl_plan *p, int64_t n_total, float *min_mean);
+sl_status launch_interp_fx(sl_plan *p, const SortBufs &b, const void *maps, const double *psi, int64_t n, const unsigned *occ,
+                           float min_mean, double *tod);
 size_t interp_f32_tiled_smem(const sl_plan *p);
 // Dynamic shared memory of the two tile-staged kernels for tile width tc.
 size_t interp_f32_tiled_smem_tc(const sl_plan *p, int tc);
@@ -470,7 +473,7 @@ size_t interp_adjoint_smem_tc(const sl_plan *p, int tc);
 // Double-float interpolation (SL_DF64 plans; k_interp_df.cu), over a sort made
 // with rec64 = 1 and with_chunks = 1.
 sl_status launch_interp_df(sl_plan *p, const SortBufs &b, int fine, const void *maps, const double *psi, int64_t n,
-                           double *tod);
+                           const unsigned *occ, float min_mean, double *tod);
 size_t interp_df_tiled_smem_tc(const sl_plan *p, int tc);
 sl_status launch_interp_adjoint_df(sl_plan *p, const SortBufs &b, int fine, const double *psi, const double *tod,
                                    int64_t n, const unsigned *occ, float min_mean, double2 *fbar);
