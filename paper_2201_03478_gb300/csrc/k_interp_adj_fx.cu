@@ -360,22 +360,42 @@ __global__ void __launch_bounds__(32 * kFaWarps, 4) k_interp_adj_fx(const __grid
 SL_CHECK_READER(chk_interp_adj_fx)
 
 // A block of four orders costs 27 mma a run of cells, whatever the run's length, so
-// k_interp_adjoint(_df) stays better where the samples leave few per occupied cell.  Equal times,
-// uniform samples: FP64 at 3.4 per cell (K = 16, 1024 x 2048 cells), 10 (K = 8, 256 x 512; K = 16
-// there: 1.43 at 7.6), 12 (K = 32, 300 x 600); DF64 at 8 (K = 16, 1024 x 2048), 30 (K = 8), 22 (K =
-// 32), 15 (K = 4, 512 x 1024).  The sort's count of occupied cells tells on the device which
-// kernel runs; the other returns at once.  The tiled kernels leave most of the chip idle on
-// small grids and small calls, where this one is always taken: at 127 x 128 cells 153 against 274 us
-// (n = 1e5, K = 4) and 79 against 115 us (3e4, K = 8; DF64 loses above 4 orders: 1.25 at K = 6, 3e5);
-// at 1024 x 2048, K = 16, 65 against 308 us (n = 1e4).  The p = 2 and 6 stencils (4 and 36 nodes) do
-// not fill rows of 16, and above 32 orders the sums no longer leave two blocks a multiprocessor.
+// k_interp_adjoint(_df) stays better where the samples leave few per occupied cell.  The sort's count of
+// occupied cells tells on the device which kernel runs; the other returns at once (4 us).  Time of the whole
+// call over the tiled kernel's, uniform samples, by grid and samples per occupied cell:
+//   127 x 128      K = 4: below 0.9 everywhere; K = 8: 1.08 at 4.5, 0.83 at 8.4; K = 16: 1.57, 1.17, 1.16, 0.89 at 4.5, 8.4, 12,
+//                  16; K = 32: 1.31, 0.97 at 24, 32 (128 tiles leave most of the chip idle in the tiled kernel)
+//   100 x 128      K <= 16: 0.43-0.97 everywhere
+//   150 x 200      K = 4: below 1 to 12, 1.2 at 24
+//   180 x 200 and 199 x 200 (one wave of tiles)   K = 4: 1.14, 1.1, 1.2, 1.15 / 0.82, 0.7 / 0.8 at 4.5, 12, 16, 24, 32; K = 16: 1.8,
+//                  1.35, 1.2, 1.17 / 0.78, 0.67; K = 1: 1.06, 1.25 at 32
+//   300 x 600      K = 4, 8, 16: 1.4 and 0.8 at 8.4 and 12; K = 5, 24: 1.18 and 0.94 at 12 and 16; K = 1: 1.06 and 0.90 at 24, 32
+//   512 x 1024     K = 4-32: 0.91-1.1 and 0.52-0.8 at 8.4 and 12; K = 1: 1.04 and 0.90 at 12 and 16
+//   DF64           180 x 200 and 199 x 200: 1.2-2.2 and 1.0-1.4 at 24 and 32; 300 x 600: 0.87-1.04 at 24 (K = 2: 1.17 at 32);
+//                  512 x 1024: 0.65-0.83 at 24 (K = 2: 1.01 at 32)
+// Small calls: the tiled kernel clears and writes whole tiles, so with 1000 to 16,000 uniform samples this
+// one takes 0.4-0.85 of its time on 300 x 600 cells and more; on 250 x 256 it is even at 4000 (1.1-1.2 at 16,000),
+// at K = 32 at 2000; on 127 x 128 0.7-1.0.  A scan of 16,000 samples, 13 to 46 per occupied cell, takes 0.3-0.9, of 40,000
+// 0.2-0.9: below 131,072 samples uniform ones reach 12 per occupied cell on the smallest grids only.
+// The p = 2 and 6 stencils (4 and 36 nodes) do not fill rows of 16, and above 32 orders the sums no
+// longer leave two blocks a multiprocessor.
 AdjRoute interp_adj_route(const sl_plan *p, int64_t n, float *min_mean) {
     const bool df = p->precision == SL_DF64;
+    const int K = p->K;
     const int64_t cells = (int64_t)(p->R + 1) * p->nphi;
-    *min_mean = df ? 24.f : 12.f;
-    if (p->p != 4 || p->K > 32) return AdjRoute::tiled;
-    if (n <= (df ? 8192 : 16384) || (cells <= 40000 && p->K <= (df ? 4 : 16)) || (double)n >= *min_mean * (double)cells) return AdjRoute::fx;
-    return AdjRoute::by_occupancy;
+    const bool large = cells >= 120000;
+    *min_mean = 0.f;
+    if (p->p != 4 || K > 32) return AdjRoute::tiled;
+    if (n <= (df || K > 16 ? 2048 : 4096) || (large && n <= (df ? 8192 : 16384))) return AdjRoute::fx;
+    if (K <= 4 && cells <= 32768 && (cells <= 20000 || n < 12 * cells)) return AdjRoute::fx;
+    if (!df && K <= 16 && (cells <= 14000 || (cells <= 20000 && n <= 16384))) return AdjRoute::fx;
+    if (n <= 16384) *min_mean = 4.f;
+    else if (n <= 131072) *min_mean = 12.f;
+    else if (df) *min_mean = large && K > 2 ? 24.f : 40.f;
+    else if (large) *min_mean = K <= 1 ? (cells < 400000 ? 30.f : 14.f) : cells < 400000 && (K == 5 || K > 16) ? 16.f : 12.f;
+    else if (cells > 20000) *min_mean = K <= 1 ? 40.f : 30.f;
+    else *min_mean = K <= 12 ? 7.f : K <= 16 ? 14.f : 32.f;
+    return (double)n >= *min_mean * (double)cells ? AdjRoute::fx : AdjRoute::by_occupancy;
 }
 
 sl_status launch_interp_adj_fx(sl_plan *p, const SortBufs &b, const double *psi, const double *tod, int64_t n, const unsigned *occ,
