@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "batchcost.cuh"
 #include "sl_internal.cuh"
 
 struct sl_batch {
@@ -33,7 +34,7 @@ struct sl_batch {
     cudaStream_t stream = nullptr;       // where the graph is captured and replayed
     bool own_stream = false;
     std::vector<sl_batch_item> items;
-    std::vector<double> cost;            // per item: measured ms (autotune) or a flop estimate
+    std::vector<double> cost;            // per item: measured (autotune) or estimated ms
     std::vector<cudaStream_t> branches;  // capture-only streams
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> joins;
@@ -491,10 +492,9 @@ sl_status sl_batch_create(sl_batch **out, const sl_batch_item *items, int nitems
     }
     if (st == SL_OK) st = cuda_check(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "fork event");
     for (int i = 0; i < nitems && st == SL_OK; ++i) st = sl_plan_reserve(b->items[i].plan, b->items[i].n);
-    for (int i = 0; i < nitems && st == SL_OK; ++i) {   // flop estimate (FP64 at 1/64 of the FP32 rate)
+    for (int i = 0; i < nitems && st == SL_OK; ++i) {
         const sl_plan *p = b->items[i].plan;
-        const double w = p->precision == SL_FP64 ? 64.0 : (p->precision == SL_DF64 ? 12.0 : 1.0);
-        b->cost[i] = w * (11.0 * (double)p->lsteps + 4.0 * 16.0 * (p->K + 1) * (double)b->items[i].n);
+        b->cost[i] = batch_cost_ms(p->precision, (double)p->lsteps, (double)(p->K + 1) * (double)b->items[i].n);
     }
     if (st == SL_OK && (flags & SL_BATCH_PERSISTENT)) {
         b->persistent = true;
