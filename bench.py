@@ -146,6 +146,26 @@ DTYPE = {"fp64": "f64", "fp32": "f32 (FP64 seeds/coords/final sum)",
          "df64": "f32x2 double-float contraction and interpolation (FP64 seeds/tables/FFT/coords)",
          "tf32x3": "f32 with a 3xTF32 tensor-core contraction (FP64 seeds/coords/final sum)"}
 PEAK_FP32_TINST = 152 * 128 * 2.07e9 / 1e12          # FP32-pipe instructions per second (x 1e12)
+PEAK_FP64_TINST = 152 * 2 * 2.07e9 / 1e12            # FP64-pipe
+PEAK_ALU_TINST = 152 * 64 * 2.07e9 / 1e12            # integer-ALU-pipe
+
+# What binds the fixed-point kernels is the pipe their scalar work runs on, not the tensor pipe: thread
+# instructions on it per recurrence step (contractions) or sample (interpolation, at 16 orders), counted by ncu
+# at lmax 512, 512 x 1024 cells, 4e6 scan samples (profiles/kernels_fixed_point_lmax512.txt).
+FX_INST = {"lcontract_fx": ("fp64pipe", 1.80), "lcontract_adj_fx": ("alupipe", 52.5),
+           "interp_fx": ("alupipe", 1549.0), "interp_adj_fx": ("alupipe", 2781.0)}
+
+FX_NOTE = {"fp64pipe": "FP64-pipe thread instructions (1.80 a recurrence step, counted by ncu); derived: 152 SMs x 2/clk x 2.07 GHz",
+           "alupipe": "integer-ALU-pipe thread instructions (counted by ncu per step or sample); derived: 152 SMs x 64/clk x 2.07 GHz"}
+
+
+def fx_inst(name, lsteps, K, n):
+    """Thread instructions of a fixed-point kernel on the pipe that binds it, and that pipe."""
+    pipe, per = FX_INST[name]
+    if name.startswith("lcontract"):
+        return per * lsteps, pipe
+    # blocks of 8 (forward) or 4 orders (transpose) beside work that does not grow with them
+    return per * float(n) * ((1 + (K + 7) // 8) / 3.0 if name == "interp_fx" else (2 + (K + 3) // 4) / 6.0), pipe
 
 
 # FP32 instructions per recurrence step of the double-float contraction
@@ -227,22 +247,20 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
     meas = {"fp64": alu.get("fp64"), "fp32": alu.get("fp32")}
     kernels = [
         (lc_name,
-         # FP64: digit products executed, 30 m16n8k8 per 32 recurrences and 8 l
-         {"fp64": 30 * 2.0 * 16 * 8 * 8 / 256 * lsteps, "fp32": fl_lc, "df64": DF_LC_INST_PER_STEP * lsteps,
+         {"fp64": fx_inst("lcontract_fx", lsteps, K, n)[0], "fp32": fl_lc, "df64": DF_LC_INST_PER_STEP * lsteps,
           # tensor work executed: 3 TF32 products x 2 flops x 16 columns (4 used, one sky)
           "tf32x3": 3 * 2.0 * 16 * lsteps}[prec],
-         {"fp64": "fp16", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "tf32"}[prec]),
+         {"fp64": "fp64pipe", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "tf32"}[prec]),
         ("interp_" + suffix, float(n) * df_interp_inst(K) if prec == "df64" else fl_in,
          {"fp64": "fp64", "fp32": "fp32", "df64": "fp32inst", "tf32x3": "fp32"}[prec]),
-        # FP64 and DF64 plans: 27 digit products per 8 orders, m16n8k16, 8 samples a group
-        ("interp_fx", float(n) * 27 * 2 * 16 * 16 * ((K + 7) // 8), "fp16"),
+        ("interp_fx",) + fx_inst("interp_fx", lsteps, K, n),
     ]
     peaks = {"fp64": (PEAK_FP64_TFLOPS, "TFLOP/s", "alu", "derived: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz"),
              "fp32": (PEAK_FP32_TFLOPS, "TFLOP/s", "alu", "derived: 152 SMs x 128 FFMA/clk x 2 flops x 2.07 GHz"),
              "fp32inst": (PEAK_FP32_TINST, "Tinst/s", "alu",
                           "derived: 152 SMs x 128 FP32 instructions/clk x 2.07 GHz (double-float arithmetic)"),
-             "fp16": (float(measured_peaks().get("bf16_tflops", 1900.0)), "TFLOP/s", "tensor",
-                      "measured bf16 burst (MEASURED_PEAKS.json); digit products of full groups"),
+             "fp64pipe": (PEAK_FP64_TINST, "Tinst/s", "alu", FX_NOTE["fp64pipe"]),
+             "alupipe": (PEAK_ALU_TINST, "Tinst/s", "alu", FX_NOTE["alupipe"]),
              "tf32": (PEAK_TF32_TFLOPS, "TFLOP/s", "tensor",
                       "measured bf16 burst (MEASURED_PEAKS.json) x nominal TF32/BF16 ratio 1.1/2.25 (of measured)")}
     roofs = {}
@@ -255,7 +273,7 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
         r = {"bound": bound, "achieved": round(ach, 4), "peak": round(peak, 4), "unit": unit,
              "frac": round(ach / peak, 4), "traffic": TRAFFIC.get((name, prec)) if traffic_ok else None,
              "avg_ms": round(avg_ms, 4),
-             ("flops_per_launch" if unit == "TFLOP/s" else "fp32_inst_per_launch"): work, "peak_note": note}
+             ("flops_per_launch" if unit == "TFLOP/s" else "inst_per_launch"): work, "peak_note": note}
         mp = meas.get(unit_kind)
         if mp:
             r["frac_of_measured_alu_peak"] = round(ach / mp, 4)
@@ -283,21 +301,19 @@ def kernel_roofs(stats, plan, prec, L, K, R, nphi, ncomp, n, alu, traffic_ok=Tru
 
 
 def adjoint_roofs(stats, plan, K, n, alu, traffic_ok=True):
-    """Adjoint kernels in fixed point on the tensor cores: the digit products of full
-    tiles (interpolation transpose: 6 + 27 ceil(K/4) m16n8k16 per 16 samples of a cell;
-    contraction transpose: 30 m16n8k16 per 32 recurrences and 16 l)."""
+    """Adjoint kernels in fixed point, against the pipe that binds them."""
     lsteps = float(plan.sizes()["lsteps"])
-    peak = float(measured_peaks().get("bf16_tflops", 1900.0))
     out = {}
-    for name, work in (("interp_adj_fx", float(n) / 16 * (6 + 27 * ((K + 3) // 4)) * 2.0 * 16 * 8 * 16),
-                       ("lcontract_adj_fx", 30 * 2.0 * 16 * 8 * 16 / 512 * lsteps)):
+    for name in ("interp_adj_fx", "lcontract_adj_fx"):
         if name in stats and stats[name][0] > 0:
+            work, pipe = fx_inst(name, lsteps, K, n)
+            peak = PEAK_FP64_TINST if pipe == "fp64pipe" else PEAK_ALU_TINST
             avg_ms = stats[name][1] / stats[name][0]
             ach = work / (avg_ms / 1e3) / 1e12
-            out[name] = {"bound": "tensor", "achieved": round(ach, 4), "peak": round(peak, 4),
-                         "unit": "TFLOP/s", "frac": round(ach / peak, 4), "avg_ms": round(avg_ms, 4),
-                         "flops_per_launch": work, "traffic": TRAFFIC.get((name, "fp64")) if traffic_ok else None,
-                         "peak_note": "measured bf16 burst (MEASURED_PEAKS.json); digit products of full tiles"}
+            out[name] = {"bound": "alu", "achieved": round(ach, 4), "peak": round(peak, 4),
+                         "unit": "Tinst/s", "frac": round(ach / peak, 4), "avg_ms": round(avg_ms, 4),
+                         "inst_per_launch": work, "traffic": TRAFFIC.get((name, "fp64")) if traffic_ok else None,
+                         "peak_note": FX_NOTE[pipe]}
     return out
 
 
@@ -795,11 +811,15 @@ def multisky_arm(args):
 # at full size for the current kernels (profiles/launches_lfi_*.txt).
 TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum per launch, LFI-like workload, 1e8 pointings
-    # (profiles/launches_lfi_{fp64,fp32,df64}.txt; single-pass ncu metrics of the current kernels)
+    # (profiles/launches_lfi_{fp64,fp32,df64}.txt; single-pass ncu metrics)
     ("lcontract_f32", "fp32"): 370.3e6 + 233.7e6,
     ("interp_f32", "fp32"): 7086.2e6 + 2115.9e6,
-    ("lcontract_df", "df64"): 672.3e6 + 511.3e6,
-    ("interp_df", "df64"): 22934.1e6 + 2736.6e6,
+    ("lcontract_df", "df64"): 673.2e6 + 512.4e6,
+    ("lcontract_fx", "fp64"): 674.2e6 + 517.4e6,
+    ("interp_fx", "fp64"): 6226.6e6 + 1246.5e6,
+    ("interp_fx", "df64"): 6231.1e6 + 1246.8e6,
+    ("interp_adj_fx", "fp64"): 6701.3e6 + 132.5e6,
+    ("lcontract_adj_fx", "fp64"): 1508.7e6 + 285.4e6,
 }
 
 
@@ -1013,10 +1033,11 @@ def sweep_arm(args):
 
 # ----------------------------------------------------------------------------- orbital dipole
 ORB_SUBSAMPLE = 20
-# FP64 flops k_orb_nodes executes per node (DADD + DMUL + 2 DFMA from an ncu op
-# count of one launch, divided by the nodes): the three library sincos and the
-# rotation and quadratic form of Eq. dipole_fast.
-ORB_NODE_FLOPS = 152     # 65 DFMA + 22 DMUL per node (ncu op counts, 1e7-sample case)
+# FP64 flops k_orb_nodes executes per node (DADD + DMUL + 2 DFMA from an ncu op count of one
+# launch, divided by the nodes): the rotation and quadratic form of Eq. dipole_fast; the sines come
+# from the integer pipe and cost six conversions on this one.
+ORB_NODE_FLOPS = 44      # 14 DFMA + 16 DMUL per node (1e7-sample case)
+ORB_SAMPLE_FLOPS = 6     # 3 DFMA per spline sample
 
 
 def orbital_inputs(n, rank):
@@ -1028,12 +1049,12 @@ def orbital_inputs(n, rank):
 
 def orbital_bytes(starts, n, s):
     """Algorithmic DRAM bytes of k_orb_eval: the 8-byte TOD write per sample, the
-    node value and second derivative (16 B) per node, and the pointing (24 B) of
-    each remainder sample evaluated exactly."""
+    cubic (32 B) per node, and the pointing (24 B) of each remainder sample evaluated
+    exactly."""
     lens = np.diff(starts)
     nodes = np.where(lens > 0, (lens - 1) // s + 1, 0)
     rem = np.maximum(lens - 1 - s * (nodes - 1), 0) * (lens > 0)
-    return 8.0 * n + 16.0 * nodes.sum() + 24.0 * rem.sum(), int(nodes.sum()), int(rem.sum())
+    return 8.0 * n + 32.0 * nodes.sum() + 24.0 * rem.sum(), int(nodes.sum()), int(rem.sum())
 
 
 def orbital_arm(args):
@@ -1114,10 +1135,10 @@ def orbital_arm(args):
     roofs = {}
     peaks = measured_peaks()
     if "orb_eval" in stats and stats["orb_eval"][0] > 0:
-        # binding roof: FP64 (one DMUL + three DFMA per spline sample, the node flops per
-        # remainder sample) ahead of HBM (the algorithmic bytes above)
+        # binding roof: FP64 (three DFMA per spline sample, the node flops per remainder
+        # sample) ahead of HBM (the algorithmic bytes above)
         avg = stats["orb_eval"][1] / stats["orb_eval"][0]
-        fl = 7.0 * (n - nrem) + ORB_NODE_FLOPS * nrem
+        fl = ORB_SAMPLE_FLOPS * (n - nrem) + ORB_NODE_FLOPS * nrem
         ach = fl / (avg / 1e3) / 1e12
         hbm = bytes_eval / (avg / 1e3) / 1e9
         roofs["orb_eval"] = {"bound": "alu", "achieved": round(ach, 4), "peak": round(PEAK_FP64_TFLOPS, 4),
@@ -1136,8 +1157,8 @@ def orbital_arm(args):
                               "traffic": TRAFFIC.get(("orb_nodes", "fp64")), "avg_ms": round(avg, 4),
                               "flops_per_launch": fl,
                               "peak_note": "FP64 pipe: unit counts x 2.07 GHz max SM clock; flops per node are "
-                                           "the FP64 operations the kernel executes (rotation with its three "
-                                           "sincos, and the quadratic form)"}
+                                           "the FP64 operations the kernel executes (rotation and quadratic "
+                                           "form; six conversions of the fixed-point sines come on top)"}
     dominant = max(stats.items(), key=lambda kv: kv[1][1])[0] if stats else None
     out = {
         "metric": "orbital dipole TOD samples/s (4pi beam; rotation every %dth sample + natural spline)" % s,
