@@ -150,7 +150,15 @@ sl_status synth_spin_maps_multi(sl_plan *plan, int nsky, const double *sky, cons
  * S_k the p-point Lagrange interpolation of F_k at (theta_i, phi_i).
  * The pointings are binned into grid tiles and sorted by a counting sort on
  * the device first; tod is written in the caller's order.  n = 0 is a no-op.
- * n < 2^31. */
+ * n < 2^31.
+ *
+ * SL_FP64 and SL_DF64 plans have several kernels for the sums.  Which one a call
+ * takes depends on the plan (orders, stencil), on n, on n per grid cell and, in
+ * DF64 plans of 13 to 16 orders, on how many cells the samples fill.  They agree to
+ * rounding (FP64 1e-15, DF64 1e-12 of the largest value), not bit for bit: a TOD
+ * evaluated in several calls can differ in the last bits from one call's.  Calls
+ * that take the same kernel give every sample the same bits; FP64 plans with the
+ * four-point stencil and 11 to 16 orders always do. */
 sl_status interp_tod(sl_plan *plan, const void *maps, const double *theta, const double *phi,
                      const double *psi, int64_t n, double *tod);
 
@@ -218,8 +226,9 @@ sl_status adjoint_synth(sl_plan *plan, const double *maps_bar, const double *sky
  * never allocates: its sort scratch is one static device array of 8.75 MiB
  * that every GPU loading the library holds until the process exits.
  *
- * Same arguments, layout and result as interp_tod (the plan is created
- * beforehand with sidelobe_plan_create).  Limits: n <= 262,144 samples per
+ * Same arguments and layout as interp_tod, and the same result to rounding (one
+ * of its kernels for every n; the plan is created beforehand with
+ * sidelobe_plan_create).  Limits: n <= 262,144 samples per
  * call (larger n returns SL_ERR_ARG: split the TOD into chunks) and plan
  * grids of at most 65,536 sort tiles (else SL_ERR_UNSUPPORTED).
  *

@@ -34,7 +34,7 @@ constexpr int kFxDig = 6, kFxSums = 8;
 // of X + bias unsigned 9-bit fields (10 bits for the first)
 constexpr unsigned long long kFxBias = (1ull << 62) + (1ull << 53) + (1ull << 44) + (1ull << 35) + (1ull << 26) +
                                        (1ull << 17) + (1ull << 8);
-// Digits for operands of twice the range: x in (-2 + 2^-7, 2 - 2^-7), X = x 2^62, d_0 within
+// Digits for operands of twice the range: x in (-2 + 2^-8, 2 - 2^-8), X = x 2^62, d_0 within
 // +-512, which FP16 and the sums above still hold (32 x (5 x 2^16 + 2^17) < 2^24).
 constexpr unsigned long long kFxBiasWide = kFxBias + (1ull << 62);
 

@@ -9,8 +9,8 @@
 //   Abar_{+m}(l) = c_l sum_pairs [y1 Ghat(N,+m) + s_l y2 (-1)^m Ghat(S,+m)]
 //   Abar_{-m}(l) = c_l sum_pairs [y2 (-1)^{m+k} Ghat(N,-m) + s_l y1 (-1)^k Ghat(S,-m)]
 // where d = c y are the rescaled recurrence values of the forward kernel, run
-// from the same FP64 start states (the evanescent zone is skipped).
-// computed by k_lcontract_adj_fx (k_adjoint_fx.cu).
+// from the same FP64 start states (the evanescent zone is skipped), computed by
+// k_lcontract_adj_fx (k_adjoint_fx.cu).
 //
 // Products (A_{k,lm} = sum_X s^X_lm conj(b^X_lk), extended to m < 0 by
 // s_{l,-m} = (-1)^m conj(s_lm)); g = d/dRe + i d/dIm:

@@ -35,7 +35,7 @@
 //      27 MMAs per 8 orders; recombination and the weighted sum over the nodes in
 //      integers, reduced over the warp by shuffles.
 // Every step is exact or rounds per sample, so a sample's value does not depend on
-// which others it is called with.
+// which others it is called with, as long as the call takes these sums (interp_route).
 // Beyond 16 orders the whole of 2 and 3 repeats per 16 orders ("block"), the phases
 // advanced by z^16 between them (that keeps every accumulator below 2^24).
 // p = 6 has 36 nodes: three row tiles, one after another; p = 2 uses 4 rows of one.

@@ -92,7 +92,7 @@ __device__ __forceinline__ void lf_store(LfWarp &W, int pr, int lane, long long 
     for (int j = 0; j < 7; ++j) o[128 * j] = d[j];
 }
 
-// The plain FP64 loop of one ring , out of line (rare).
+// The plain FP64 loop of one ring, out of line (rare).
 __device__ __noinline__ void lf_plain(const LcArgs &a, int m, int k, int pair, int neg) {
     if (pair >= a.npairs) return;
     const int64_t moff = (int64_t)m * (2 * a.L + 1 - m) / 2, si = start_index(a, k, m, neg, pair);
@@ -301,7 +301,7 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
                 lf_columns(a, moff, m, k, l, t.c, v[h]);
             }
             W.cd[i] = make_double2(t.a, -t.b);
-            bool big;                   // the batch's FP64 steps cover these (a' falls with l)
+            bool big;                   // the batch's FP64 steps cover these (a' + |b'| falls over every second l)
             W.ci[i] = lf_coef(t.a, t.b, big);
             steep |= (uint64_t)__ballot_sync(0xffffffffu, big) << (32 * h);
 #pragma unroll

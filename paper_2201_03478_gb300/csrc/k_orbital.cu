@@ -13,8 +13,8 @@
 // Kernels (all FP64):
 //   k_orb_moments  one thread: the nine moments from b_lk, l <= 2
 //   k_orb_nodes    one thread per spline node: Eq. dipole_fast at that sample
-//   k_orb_spline   one CTA per pointing period: the cubics of the natural spline
-//                  through the period's nodes
+//   k_orb_spline   one CTA per pointing period (a warp for short ones): the cubics of
+//                  the natural spline through the period's nodes
 //   k_orb_eval     one thread per sample: the cubic between nodes, Eq.
 //                  dipole_fast after the last node (or everywhere when s = 1)
 // All are bound by the FP64 pipe (2 operations a clock and SM), so they keep its work
@@ -46,7 +46,6 @@ constexpr int kOrbEvalPerThread = 8;   // samples per thread of k_orb_eval
 constexpr int kOrbRun = 8;             // rows per thread and sweep round of k_orb_spline
 constexpr int kOrbPivots = 40;         // pivots tabulated; the last one is the limit
 
-// Eq. dipole_fast at one sample.  beta' = Rz(-psi) Ry(-theta) Rz(-phi) beta.
 // x 2^-62, x = 0 or |x| >= 1: the exponent lowered by integer arithmetic
 __device__ __forceinline__ double orb_q62(long long x) {
     const double v = (double)x;
@@ -62,6 +61,7 @@ __device__ __forceinline__ void orb_sincos(double x, const longlong2 *tab, doubl
     }
 }
 
+// Eq. dipole_fast at one sample.  beta' = Rz(-psi) Ry(-theta) Rz(-phi) beta.
 __device__ __forceinline__ double orb_value(const longlong2 *tab, const double *__restrict__ S, double T0, double q,
                                             double th, double ph, double ps, const double *__restrict__ b) {
     double st, ct, sp, cp, ss, cs;

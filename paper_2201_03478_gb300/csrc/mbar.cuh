@@ -63,12 +63,12 @@ __device__ __forceinline__ void mbar_arrive_cp_async(uint32_t bar) {
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst)), "l"(src) : "memory");
 }
-// 8-byte copy; with ok == false nothing is read and the destination is zero-filled
 // 16-byte copy through L1; with ok == false nothing is read and the destination is zero-filled
 __device__ __forceinline__ void cp_async16z(void *dst, const void *src, bool ok) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" :: "r"(smem_u32(dst)), "l"(src), "r"(ok ? 16 : 0)
                  : "memory");
 }
+// 8-byte copy; with ok == false nothing is read and the destination is zero-filled
 __device__ __forceinline__ void cp_async8(void *dst, const void *src, bool ok) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(smem_u32(dst)), "l"(src), "r"(ok ? 8 : 0)
                  : "memory");

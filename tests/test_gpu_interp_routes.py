@@ -40,3 +40,27 @@ def test_df64_by_samples_per_occupied_cell(K, n, ncells, fixed):
     got, want = sl.interp_tod(plan, maps, *t), sl.interp_tod(ref, maps, *t)
     assert torch.equal(got, want) == fixed
     assert float((got - want).abs().max()) <= 1e-11 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("K,n", [(4, 20480), (8, 20480)])
+def test_values_across_the_switch_by_size(K, n):
+    """One sample more takes another kernel: same values to rounding (both forms' bound of the direct
+    comparison, 16 (K + 1)^2 2^-53 of the largest |F| at sum |w| <= 2); on the same side, same bits."""
+    sl, plan = _plan(K, 200, 400, "fp64")
+    maps, t = _cube(K, 200, 400), _points(n + 1, 0)
+    more = sl.interp_tod(plan, maps, *t)
+    few = sl.interp_tod(plan, maps, *(a[:n].contiguous() for a in t))
+    less = sl.interp_tod(plan, maps, *(a[:n - 7000].contiguous() for a in t))
+    top = float(torch.view_as_real(maps).abs().max())
+    assert not torch.equal(more[:n], few)
+    assert float((more[:n] - few).abs().max()) <= 16.0 * (K + 1) ** 2 * 2.0 ** -53 * 2.0 * top
+    assert torch.equal(few[:n - 7000], less)
+
+
+@pytest.mark.parametrize("n", [300, 30000, 400000])
+def test_eleven_to_sixteen_orders_have_one_value(n):
+    """FP64, four-point stencil: the same bits in calls of any size."""
+    sl, plan = _plan(12, 200, 400, "fp64")
+    maps, t = _cube(12, 200, 400), _points(500000, 0)
+    whole = sl.interp_tod(plan, maps, *t)
+    assert torch.equal(sl.interp_tod(plan, maps, *(a[:n].contiguous() for a in t)), whole[:n])
