@@ -949,6 +949,13 @@ SWEEP = [(256, 0), (256, 10), (512, 0), (512, 10), (1024, 0), (1024, 10), (2048,
          (4096, 10), (8192, 0), (8192, 10), (512, 100)]
 
 
+def sweep_fraction(prec, lsteps, ms):
+    """Fraction of the FP32 peak of an FP32 plan's contraction, 11 flops a visited step.  None for FP64 plans: their sums
+    are integer digits on the tensor cores, and the FP64 pipe's instructions a step (the growing part of the
+    recurrence) change with lmax and kmax; nor for DF64 plans."""
+    return 11.0 * lsteps / (ms / 1e3) / 1e12 / PEAK_FP32_TFLOPS if prec == "fp32" and ms else None
+
+
 def sweep_arm(args):
     """Cube-build runtime against lmax (the paper's Fig. speed): random sky, an
     elliptical-Gaussian-like beam with kmax (the paper's m_max) 0 or 10, lmax 256 ... 8192
@@ -1002,9 +1009,9 @@ def sweep_arm(args):
             pt = {"lmax": L, "kmax": K, "nrings": R, "nphi": nphi, "precision": prec, "ms": round(ms, 3),
                   "plan_s": round(t_plan, 2), "dense_flops": dense, "executed_flops": 11.0 * lsteps,
                   "kernel_ms": {k: round(v[1] / steps, 3) for k, v in stats.items()}}
-            if lc_ms and prec in ("fp64", "fp32"):
-                peak = PEAK_FP64_TFLOPS if prec == "fp64" else PEAK_FP32_TFLOPS
-                pt["lcontract_frac_of_peak"] = round(11.0 * lsteps / (lc_ms / 1e3) / 1e12 / peak, 4)
+            frac = sweep_fraction(prec, lsteps, lc_ms)
+            if frac is not None:
+                pt["lcontract_frac_of_peak"] = round(frac, 4)
             points.append(pt)
             print("sweep lmax=%d kmax=%d %s: %.2f ms (plan %.1f s)" % (L, K, prec, ms, t_plan), file=sys.stderr,
                   flush=True)

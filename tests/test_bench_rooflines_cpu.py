@@ -21,3 +21,9 @@ def test_orbital_kernels():
     assert 0.5 < bench.ORB_SAMPLE_FLOPS * 1e8 / 0.681e-3 / 1e12 / bench.PEAK_FP64_TFLOPS < 0.9
     import numpy as np
     assert bench.orbital_bytes(np.array([0, 41, 61]), 61, 20)[0] == 8 * 61 + 32 * 4 + 24 * 19
+
+
+def test_sweep_fractions():
+    # lmax 4096, kmax 10: 2.5e11 steps; the FP64 plans' 1.0 s would be 2.2 of the FP64 peak, which their sums do not use
+    assert bench.sweep_fraction("fp64", 2.5e11, 1009.0) is None and bench.sweep_fraction("df64", 2.5e11, 746.0) is None
+    assert 0.0 < bench.sweep_fraction("fp32", 2.5e11, 69.2) < 0.79
