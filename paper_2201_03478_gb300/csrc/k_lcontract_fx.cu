@@ -34,10 +34,11 @@
 // largest value; the digit sums are read out after each batch (64 l keep |acc| < 2^24) and
 // added in FP64.
 //
-// A batch with a non-finite V, or one above 2^960, sends the whole unit to the plain FP64 loop (the sums
-// then overflow or turn NaN where that form does).  One whose largest V is below 2^-959 (the tail of a
-// Gaussian beam: exp(-l^2 / 2 sigma^2) from l = 36 sigma on) is summed times 2^600: in the plain loop,
-// lmax 2048, kmax 32 with such a beam took 1968 ms, 981 in the FP64 form, 409 so.
+// A batch with a non-finite V, or one above 2^960, sends the whole unit to the plain FP64 loop (the
+// sums then overflow or turn NaN where that form does).  One whose largest V is below 2^-959 (the
+// tail of a Gaussian beam: exp(-l^2 / 2 sigma^2) from l = 36 sigma on) is summed times 2^600, unless sums
+// above 2^400 stand there already: in the plain loop, lmax 2048, kmax 32 with such a beam took
+// 1968 ms, 981 in the FP64 form, 401 so.
 #include <algorithm>
 
 #include "lcontract.cuh"
@@ -47,7 +48,6 @@ namespace sl {
 
 constexpr int kLfWarps = 4;        // warps per CTA, four CTAs per SM (128 registers a thread)
 constexpr int kLfBatch = 64;       // l per batch
-constexpr int kLfTiny = 1 << 11;   // added to a batch's exponent field: V is held times 2^600
 
 struct LfWarp {                    // one warp's shared memory
     uint32_t yd[7][4][32];         // digits of y at 8 l: [digit][pair of l][ring], swizzled (lf_slot)
@@ -215,8 +215,7 @@ __device__ __forceinline__ void lf_batch(const LcArgs &a, LfWarp &W, int grp, bo
     const int h0 = odd ? 1 << 9 : 1 << 18, h1 = odd ? 1 : 1 << 9, h2 = odd ? 0 : 1;
     const int w2 = odd ? 1 << 27 : 0, w3 = odd ? 1 << 18 : 1 << 27, w4 = odd ? 1 << 9 : 1 << 18, w5 = odd ? 1 : 1 << 9,
               w6 = odd ? 0 : 1;
-    // 2^(U + e - 34), e = escale - 1022
-    const double sc = __longlong_as_double((long long)((escale & (kLfTiny - 1)) + U + 1 - 34) << 52);
+    const double sc = __longlong_as_double((long long)(escale + U + 1 - 34) << 52);     // 2^(U + e - 34), e = escale - 1022
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
         long long H[4], Lw[4];
@@ -234,15 +233,25 @@ __device__ __forceinline__ void lf_batch(const LcArgs &a, LfWarp &W, int grp, bo
             const long long h = (odd ? H[2 + e] : H[e]) + __shfl_xor_sync(0xffffffffu, odd ? H[e] : H[2 + e], 2);
             const long long l = (odd ? Lw[2 + e] : Lw[e]) + __shfl_xor_sync(0xffffffffu, odd ? Lw[e] : Lw[2 + e], 2);
             double &o = e ? s.y : s.x;
-            if (escale < kLfTiny) {
-                o = fma((double)l, sc * 0x1p-36, o);
-                o = fma((double)h, sc, o);
-            } else {
-                o = fma(fma((double)h, sc, (double)l * (sc * 0x1p-36)), 0x1p-600, o);
-            }
+            o = fma((double)l, sc * 0x1p-36, o);
+            o = fma((double)h, sc, o);
         }
         W.sum[grp][t][lane] = s;
     }
+}
+
+// This lane's sums times f, for a batch of tiny V; false, in every lane, if one would overflow.  Out of line
+// (rare): 2^600 applied as the sums are read out cost every batch 2% of the kernel.
+__device__ __noinline__ bool lf_scale_sums(LfWarp &W, int groups, double f) {
+    const int lane = threadIdx.x & 31;
+    bool ok = true;
+    for (int grp = 0; grp < groups; ++grp)
+        for (int t = 0; t < 2; ++t) {
+            double2 &s = W.sum[grp][t][lane];
+            ok = ok && fabs(s.x) < 0x1p400 && fabs(s.y) < 0x1p400;
+            s = make_double2(s.x * f, s.y * f);
+        }
+    return __all_sync(0xffffffffu, ok);
 }
 
 // One unit: (m, k, 16 groups ring pairs); 2 groups (V staged once for both) or 1.
@@ -317,11 +326,8 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
         }
         mx = __reduce_max_sync(0xffffffffu, mx);
         int escale = (int)(mx >> 20);   // exponent field of the largest |V|
-        if (escale > 1983) {
-            for (int grp = 0; grp < groups; ++grp) lf_plain(a, m, k, base + 16 * grp + (lane & 15), neg);
-            return;
-        }
-        if (escale < 64) {              // all zero (any scale), or too small for one: times 2^600
+        bool plain = escale > 1983, tiny = false;
+        if (escale < 64) {              // all zero (any scale), or too small for one: V and the sums times 2^600
             mx = 0;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
@@ -331,9 +337,14 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
                     mx = max(mx, (uint32_t)__double2hiint(v[h][c]) & 0x7fffffffu);
                 }
             escale = (int)(__reduce_max_sync(0xffffffffu, mx) >> 20);
-            escale = escale ? escale | kLfTiny : 64;
+            tiny = escale > 0;
+            escale = max(escale, 64);
+            if (tiny) plain = !lf_scale_sums(W, groups, 0x1p600);
         }
-        const int ef = escale & (kLfTiny - 1);
+        if (plain) {
+            for (int grp = 0; grp < groups; ++grp) lf_plain(a, m, k, base + 16 * grp + (lane & 15), neg);
+            return;
+        }
         // digits, to the B fragment of each 8 l: element (l, column n), n = digit parity * 4 + c, in
         // lane 4 n + (l % 8) / 2, half l % 2
 #pragma unroll
@@ -343,7 +354,7 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
 #pragma unroll
             for (int c = 0; c < 4; c += 2) {
                 uint32_t d[kFxDig];
-                fx_digits(fx_from_double(v[h][c], ef), fx_from_double(v[h][c + 1], ef), d);
+                fx_digits(fx_from_double(v[h][c], escale), fx_from_double(v[h][c + 1], escale), d);
 #pragma unroll
                 for (int j = 0; j < kFxDig; ++j) {
                     const int ln = 4 * ((j & 1) * 4 + c);
@@ -363,6 +374,7 @@ __device__ __forceinline__ void lf_unit(const LcArgs &a, LfWarp &W, int groups, 
             if (grp) fixed1 = fixed;
             else fixed0 = fixed;
         }
+        if (tiny) lf_scale_sums(W, groups, 0x1p-600);
     }
     __syncwarp();
     for (int grp = 0; grp < groups; ++grp)

@@ -48,3 +48,14 @@ def test_products_below_the_scales(L, K, R, e):
     # results below 2^-1022 are rounded to 2^-1074: (e + 1074) bits after the point
     floor = 2.0 ** (-1074 - e) * np.sqrt(want.numel()) * 4 * L
     assert float(torch.linalg.norm(got - want)) <= L * L * 2.0 ** -52 * float(torch.linalg.norm(want)) + floor
+
+
+@pytest.mark.parametrize("L,K,R", [(130, 3, 40), (130, 40, 97)])
+def test_a_tail_behind_large_sums(L, K, R):
+    """From 2^460 to zero within a unit: sums that 2^600 would carry past the largest double."""
+    cube, beam = _setup(L, K, R)
+    beam = beam * np.exp2(np.maximum(460.0 - 16.0 * np.arange(L + 1), -1100.0))
+    a, b = (torch.view_as_real(cube(v)) for v in (beam, np.where(np.abs(beam) < 1e-250, 0, beam)))
+    assert bool(torch.isfinite(a).all())
+    a, b = a * 2.0 ** -400, b * 2.0 ** -400
+    assert float(torch.linalg.norm(a - b)) <= L * L * 2.0 ** -52 * float(torch.linalg.norm(b))
