@@ -20,8 +20,8 @@
 // only the columns that leave the stencil are added to the cube (atomically), a quarter of the
 // values when the next cell is the next column.
 //
-// Measured (before -> after): 5e6 scanning samples at K = 16, 1024 x 2048 cells 7.62 -> 1.46 ms;
-// 2e7 uniform ones there 28.5 -> 15.9 ms (9.5 a cell); 1e7 at K = 4, 127 x 128 cells 5.21 -> 1.86 ms.
+// Measured (before -> after): 5e6 scanning samples at K = 16, 1024 x 2048 cells 7.62 -> 1.47 ms;
+// 2e7 uniform ones there 28.5 -> 16.0 ms (9.5 a cell); 1e7 at K = 4, 127 x 128 cells 5.21 -> 1.83 ms.
 // Bound by issue and the integer pipe (54% and 46% of their rates at 48 samples a cell, K = 16,
 // with 2.8 warps a scheduler): digits of 16 nodes and 2 K + 1 phases a sample, recombination a run.
 //
@@ -371,8 +371,12 @@ SL_CHECK_READER(chk_interp_adj_fx)
 //                  1.35, 1.2, 1.17 / 0.78, 0.67; K = 1: 1.06, 1.25 at 32
 //   300 x 600      K = 4, 8, 16: 1.4 and 0.8 at 8.4 and 12; K = 5, 24: 1.18 and 0.94 at 12 and 16; K = 1: 1.06 and 0.90 at 24, 32
 //   512 x 1024     K = 4-32: 0.91-1.1 and 0.52-0.8 at 8.4 and 12; K = 1: 1.04 and 0.90 at 12 and 16
+//   724 x 1500     K = 4-32: 1.14-1.32, 0.87-1.01 and 0.73-0.82 at 3, 5, 7; K = 2: 0.95 at 7; K = 1: 0.99 at 12
+//   1024 x 2048 to 2048 x 4096   K = 4-32: 0.84-1.16 and 0.67-0.90 at 3 and 5; K = 2: 0.77-0.85 at 7; K = 1: 0.73-0.86 at 12
+//   the same, 4 to 10 samples in each of 3% or 30% of the cells: K = 2 to 32 0.40-0.91
 //   DF64           180 x 200 and 199 x 200: 1.2-2.2 and 1.0-1.4 at 24 and 32; 300 x 600: 0.87-1.04 at 24 (K = 2: 1.17 at 32);
-//                  512 x 1024: 0.65-0.83 at 24 (K = 2: 1.01 at 32)
+//                  512 x 1024: 0.65-0.83 at 24 (K = 2: 1.01 at 32); 724 x 1500 and more: K = 4-16 1.06-1.33 and 0.61-0.90
+//                  at 7 and 12; K = 32 0.83-0.95 at 16
 // Small calls: the tiled kernel clears and writes whole tiles, so with 1000 to 16,000 uniform samples this
 // one takes 0.4-0.85 of its time on 300 x 600 cells and more; on 250 x 256 it is even at 4000 (1.1-1.2 at 16,000),
 // at K = 32 at 2000; on 127 x 128 0.7-1.0.  A scan of 16,000 samples, 13 to 46 per occupied cell, takes 0.3-0.9, of 40,000
@@ -383,7 +387,7 @@ AdjRoute interp_adj_route(const sl_plan *p, int64_t n, float *min_mean) {
     const bool df = p->precision == SL_DF64;
     const int K = p->K;
     const int64_t cells = (int64_t)(p->R + 1) * p->nphi;
-    const bool large = cells >= 120000;
+    const bool large = cells >= 120000, huge = cells >= 1000000;
     *min_mean = 0.f;
     if (p->p != 4 || K > 32) return AdjRoute::tiled;
     if (n <= (df || K > 16 ? 2048 : 4096) || (large && n <= (df ? 8192 : 16384))) return AdjRoute::fx;
@@ -391,6 +395,8 @@ AdjRoute interp_adj_route(const sl_plan *p, int64_t n, float *min_mean) {
     if (!df && K <= 16 && (cells <= 14000 || (cells <= 20000 && n <= 16384))) return AdjRoute::fx;
     if (n <= 16384) *min_mean = 4.f;
     else if (n <= 131072) *min_mean = 12.f;
+    else if (huge && K > 2) *min_mean = !df ? 5.f : K <= 16 ? 12.f : 16.f;
+    else if (huge && K == 2 && !df) *min_mean = 7.f;
     else if (df) *min_mean = large && K > 2 ? 24.f : 40.f;
     else if (large) *min_mean = K <= 1 ? (cells < 400000 ? 30.f : 14.f) : cells < 400000 && (K == 5 || K > 16) ? 16.f : 12.f;
     else if (cells > 20000) *min_mean = K <= 1 ? 40.f : 30.f;
