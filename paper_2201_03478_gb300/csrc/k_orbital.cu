@@ -13,8 +13,9 @@
 // Kernels (all FP64):
 //   k_orb_moments  one thread: the nine moments from b_lk, l <= 2
 //   k_orb_nodes    one thread per spline node: Eq. dipole_fast at that sample
-//   k_orb_spline   one CTA per pointing period (a warp for short ones): the cubics of
-//                  the natural spline through the period's nodes
+//   k_orb_spline   one CTA per pointing period (a warp for short ones, k_orb_spline_tiny's
+//                  threads for the shortest): the cubics of the natural spline through
+//                  the period's nodes
 //   k_orb_eval     one thread per sample: the cubic between nodes, Eq.
 //                  dipole_fast after the last node (or everywhere when s = 1)
 // All are bound by the FP64 pipe (2 operations a clock and SM), so they keep its work
@@ -146,8 +147,8 @@ __global__ void __launch_bounds__(256) k_orb_nodes(const OrbArgs a) {
 // rows (8 l + i) fall on distinct banks
 __device__ __forceinline__ int orb_pad(int q) { return q + (q >> 3); }
 // threads per period: one warp up to kOrbShortNodes nodes (one round of it), eight beyond.  A short
-// period leaves most of eight warps at barriers: 1e7 samples in periods of 100 (5 nodes, s = 20) 1181 -> 348
-// us, of 1950 (98 nodes) 97 -> 51, of 4000 (200 nodes) 58 -> 30.
+// period leaves most of eight warps at barriers: 1e7 samples in periods of 1950 (98 nodes, s = 20) 97 -> 51
+// us, of 4000 (200 nodes) 58 -> 30.  The shortest: k_orb_spline_tiny.
 constexpr int kOrbThreads = 256, kOrbShortThreads = 32;
 
 // The value that enters this thread's rows, from every thread's (end value from zero A, factor F)
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(NT) k_orb_spline(const OrbArgs a) {
     __shared__ double s_end[2][NT / 32];
     const int64_t p = blockIdx.x;
     const int64_t g0 = a.noff[p], M = a.noff[p + 1] - g0;
-    if (M < 2 || (M <= kOrbShortNodes) != (NT == kOrbShortThreads)) return;     // nothing to do, or the other launch's
+    if (M <= kOrbTinyNodes || (M <= kOrbShortNodes) != (NT == kOrbShortThreads)) return;    // nothing to do, or another launch's
     for (int j = threadIdx.x; j < kOrbPivots; j += NT) s_piv[j] = a.piv[j];
     __syncthreads();
     const double *__restrict__ y = a.y + g0;
@@ -257,6 +258,42 @@ __global__ void __launch_bounds__(NT) k_orb_spline(const OrbArgs a) {
         const double m1 = above;                     // node 0: N_0 = 0, N_1 (0 when there are two nodes)
         cub[0] = make_double4_32a(y[0], (y[1] - y[0]) - m1, 0.0, m1);
     }
+}
+
+// The same for periods of 2 to kOrbTinyNodes nodes, a thread each, row by row: in a warp of its own such a
+// period leaves most lanes of every FP64 instruction empty: 5e6 samples in periods of 50, s = 7 (8 nodes) 564 ->
+// 22 us, of 200, s = 12 (17 nodes) 180 -> 18; at 25 nodes 1e6 samples take the warp form's 77 us.
+constexpr int kOrbTinyThreads = 128;
+
+__global__ void __launch_bounds__(kOrbTinyThreads) k_orb_spline_tiny(const OrbArgs a) {
+    static_assert(kOrbTinyNodes <= kOrbPivots, "pivots tabulated");
+    __shared__ double s_piv[kOrbPivots], s_dp[kOrbTinyNodes][kOrbTinyThreads];
+    for (int j = threadIdx.x; j < kOrbPivots; j += kOrbTinyThreads) s_piv[j] = a.piv[j];
+    __syncthreads();
+    const int64_t p = (int64_t)blockIdx.x * kOrbTinyThreads + threadIdx.x;
+    if (p >= a.nper) return;
+    const int64_t g0 = a.noff[p];
+    if (a.noff[p + 1] - g0 < 2 || a.noff[p + 1] - g0 > kOrbTinyNodes) return;
+    const int M = (int)(a.noff[p + 1] - g0);
+    const double *__restrict__ y = a.y + g0;
+    double4_32a *cub = a.cub + g0;
+    double d = 0.0, y0 = y[0], y1 = y[1];
+    for (int j = 1; j <= M - 2; ++j) {
+        const double y2 = y[j + 1];
+        d = (y2 - 2.0 * y1 + y0 - d) * s_piv[j];
+        s_dp[j][threadIdx.x] = d;
+        y0 = y1;
+        y1 = y2;
+    }
+    double m1 = 0.0;                                 // N of the row above; y0, y1: nodes M - 2 and M - 1
+    for (int j = M - 2; j >= 1; --j) {
+        const double m0 = s_dp[j][threadIdx.x] - s_piv[j] * m1;
+        cub[j] = make_double4_32a(y0, (y1 - y0) - fma(2.0, m0, m1), 3.0 * m0, m1 - m0);
+        m1 = m0;
+        y1 = y0;
+        y0 = y[j - 1];
+    }
+    cub[0] = make_double4_32a(y0, (y1 - y0) - m1, 0.0, m1);
 }
 
 __global__ void __launch_bounds__(256) k_orb_eval(const OrbArgs a) {
@@ -338,6 +375,8 @@ sl_status launch_orbital(sl_plan *p, const OrbLaunch &o) {
         sl_status st = cuda_check(cudaGetLastError(), "k_orb_nodes launch");
         if (st != SL_OK) return st;
         slot = timing_begin(p, "orb_spline");
+        if (o.ntiny > 0)
+            k_orb_spline_tiny<<<(unsigned)((a.nper + kOrbTinyThreads - 1) / kOrbTinyThreads), kOrbTinyThreads, 0, p->stream>>>(a);
         if (o.nshort > 0) k_orb_spline<kOrbShortThreads><<<(unsigned)a.nper, kOrbShortThreads, 0, p->stream>>>(a);
         if (o.nlong > 0) k_orb_spline<kOrbThreads><<<(unsigned)a.nper, kOrbThreads, 0, p->stream>>>(a);
         timing_end(p, slot);

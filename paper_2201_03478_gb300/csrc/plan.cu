@@ -1081,7 +1081,7 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     for (int j = 1; j < kPiv; ++j) piv[j] = 1.0 / (4.0 - piv[j - 1]);
     for (int r = 0; r <= subsample; ++r) wt[r] = (double)r / (double)subsample;
     noff[0] = 0;
-    int64_t nshort = 0, nlong = 0;
+    int64_t ntiny = 0, nshort = 0, nlong = 0;
     for (int64_t k = 0; k < nper; ++k) {
         const int64_t np = period_start[k + 1] - period_start[k];
         if (np < 0) return set_error(SL_ERR_ARG, "orbital_dipole_tod: period_start decreases at period %lld", (long long)k);
@@ -1090,7 +1090,8 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
         start[k] = period_start[k];
         const int64_t nodes = subsample > 1 && np > 0 ? (np - 1) / subsample + 1 : 0;
         noff[k + 1] = noff[k] + nodes;
-        nshort += nodes > 1 && nodes <= kOrbShortNodes;
+        ntiny += nodes > 1 && nodes <= kOrbTinyNodes;
+        nshort += nodes > kOrbTinyNodes && nodes <= kOrbShortNodes;
         nlong += nodes > kOrbShortNodes;
         for (int c = 0; c < 3; ++c) {
             bet[3 * k + c] = beta[3 * k + c];
@@ -1126,6 +1127,7 @@ sl_status orbital_dipole_tod(sl_plan *p, const double *beam, double T0, double q
     o.n = n;
     o.nper = nper;
     o.nnodes = nnodes;
+    o.ntiny = ntiny;
     o.nshort = nshort;
     o.nlong = nlong;
     o.s = subsample;

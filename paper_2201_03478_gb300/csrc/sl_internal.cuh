@@ -378,7 +378,7 @@ void timing_end(sl_plan *p, int idx);
 inline int64_t sky_row_stride(int64_t nalm) { return (nalm + 1) & ~(int64_t)1; }
 
 // orbital dipole (k_orbital.cu): device pointers of one call
-constexpr int64_t kOrbShortNodes = 256;
+constexpr int64_t kOrbTinyNodes = 24, kOrbShortNodes = 256;
 struct OrbLaunch {
     const double *theta, *phi, *psi;
     const int64_t *start, *noff;
@@ -387,7 +387,7 @@ struct OrbLaunch {
     const double *frac;      // [s + 1] position between nodes r / s
     double T0, q;
     int64_t n, nper, nnodes;
-    int64_t nshort, nlong;   // periods of 2 .. kOrbShortNodes nodes, and of more
+    int64_t ntiny, nshort, nlong;   // periods of 2 .. kOrbTinyNodes nodes, .. kOrbShortNodes, and of more
     int s;
     double *y, *cub, *tod;   // cub: [nnodes][4], 32-byte aligned
     int accumulate;
